@@ -1,5 +1,6 @@
-// FP64 form of the two-fluid spin-SPH step (every stored field and every
-// arithmetic operation in double precision).
+// FP64 form of the two-fluid spin-SPH step: every stored field in double
+// precision; the neighbour passes in 62-bit fixed point where that holds more
+// than a double does (sph_fixed.cuh), everything else in double precision.
 //
 // Model (Sec. 2.1, Eqs. 1, 2, 4; Algorithm 1; Sec. 3 boundary set-up):
 //   density   rho_i = sum_j m_j W_ij (self included), Wendland C2, support 2h,
@@ -25,6 +26,8 @@
 
 namespace sphgb {
 namespace {
+
+using fx::u64;
 
 __device__ __forceinline__ void latch(uint32_t* err, uint32_t bit) {
   if ((*(volatile uint32_t*)err & bit) == 0u) atomicOr(err, bit);
@@ -159,7 +162,8 @@ __global__ void k_kick_fp64(int64_t n, Fp64Buf b, Fp64Fields f,
 
 // -------------------------------------------------------------------- reorder
 
-__global__ void k_reorder_fp64(int64_t n, Fp64Buf src, Fp64Buf dst, CellWs cw, NbrWs nw) {
+__global__ void k_reorder_fp64(int64_t n, Fp64Buf src, Fp64Buf dst, CellWs cw, NbrWs nw,
+                               const InstDev* __restrict__ inst) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t j = checked_index(cw.perm[k], n, cw.err);
@@ -172,6 +176,16 @@ __global__ void k_reorder_fp64(int64_t n, Fp64Buf src, Fp64Buf dst, CellWs cw, N
     dst.inst[k] = src.inst[j];
     cw.skey[k] = cw.key[j];
     nw.posf[k] = make_float4((float)p.x, (float)p.y, (float)p.z, (float)p.w);
+    const fx::Unit U = inst[src.inst[j]].fx_unit;
+    QPos q;
+    q.x = fx::to_fixed(p.x, U);
+    q.y = fx::to_fixed(p.y, U);
+    q.z = fx::to_fixed(p.z, U);
+    q.tag = (uint32_t)p.w;
+    q.exps = 0u;
+    nw.posq[k] = q;
+    // a wall placed from a non-finite reference (fluid is tested at its drift)
+    if (!finite3(p.x, p.y, p.z)) latch(cw.err, ERR_NONFINITE);
   }
 }
 
@@ -205,34 +219,6 @@ __device__ __forceinline__ int z_wrap(uint32_t ent, int cz_i, int nz) {
   return (cz_i == 0 && cz == 2u) ? 1 : ((cz_i == nz - 1 && cz == 0u) ? -1 : 0);
 }
 
-// ------------------------------------------------- square roots of distances
-
-// sqrt(x) for the pair distances of the density pass, with few FP64
-// instructions (the FP64 pipe bounds that pass).  The FP32 hardware
-// estimate of 1/sqrt(x) is taken on the top 20 mantissa bits of x;
-// operand and estimate move between the formats by integer operations on
-// their bits, so no conversion instruction is issued.  One step of the
-// third-order iteration y <- y + y e (1/2 + 3e/8), e = 1 - x y^2 (the first
-// terms of the binomial series (1 - e)^(-1/2) = 1 / (y sqrt(x))) takes the
-// estimate's relative error, below 2^-19, to about (5/16) |e|^3 < 2^-55:
-// x times the refined 1/sqrt(x) is within about an ulp of sqrt(x).  An
-// argument whose FP32 form would not be normal (zero, tiny, huge) takes
-// CUDA's sqrt.
-__device__ __forceinline__ bool fp32_range(int hi) {
-  return hi >= 0x38100000 && hi < 0x47F00000;  // 2^-126 <= x < 2^128
-}
-__device__ __forceinline__ double rsqrt_seed_step(double x, int hi) {
-  const float xf = __int_as_float((int)(((unsigned)hi - (896u << 20)) << 3));
-  const unsigned yb = (unsigned)__float_as_int(rsqrtf(xf));
-  const double y = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-__device__ __forceinline__ double sqrt_dist(double x) {
-  const int hi = __double2hiint(x);
-  return fp32_range(hi) ? x * rsqrt_seed_step(x, hi) : sqrt(x);
-}
-
 // -------------------------------------------------------------------- density
 
 __device__ __forceinline__ double ipow(double x, int e) {
@@ -241,17 +227,51 @@ __device__ __forceinline__ double ipow(double x, int e) {
   return r;
 }
 
+// The FP64 route of a candidate pair whose fixed-point r^2 does not decide it
+// (within rounding of the cutoff, or nearly coincident): the exact test
+// r^2 < (2h)^2 without fused multiply-adds, strict <, and the W shape
+// t^4 (2q + 1) of a neighbour; -1 for a pair outside.
+__device__ __noinline__ double exact_pair_shape(const dvec4* pos, uint32_t i, uint32_t j, int wz,
+                                                const InstDev* P) {
+  const dvec4 a = pos[i], b = pos[j];
+  const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
+  double dz = __dsub_rn(a.z, b.z);
+  if (wz > 0) dz = __dadd_rn(dz, P->Hz);
+  else if (wz < 0) dz = __dsub_rn(dz, P->Hz);
+  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+  if (!(r2 < P->cut2)) return -1.0;
+  const double r = sqrt(r2);
+  const double t1 = fma(-0.5 * P->inv_h, r, 1.0), t2 = t1 * t1;
+  return t2 * t2 * fma(2.0 * P->inv_h, r, 1.0);
+}
+
+// A QPos record in one 256-bit load.
+__device__ __forceinline__ QPos ld_qpos(const QPos* q) {
+  unsigned long long x, y, z, s;
+  asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(x), "=l"(y), "=l"(z), "=l"(s) : "l"(q));
+  QPos r;
+  r.x = (int64_t)x;
+  r.y = (int64_t)y;
+  r.z = (int64_t)z;
+  r.tag = (uint32_t)s;
+  r.exps = (uint32_t)(s >> 32);
+  return r;
+}
+
 // Density and Tait pressure (Eq. 4), one thread per particle, from the hit
 // bits of the FP32 prefilter of the neighbour search (sph_search.cu): every
-// candidate whose bit is set is re-tested exactly in FP64 (no fused
-// multiply-add in r^2, strict <); the neighbours are summed and written as
-// i's neighbour list for the pair pass, a fluid particle's inviscid
-// neighbours first (in candidate order, count_a of them) and then the others
-// (in candidate order, from a second walk over the bits set aside for them).
-// The walk takes 4 candidates at a time: their table entries, then their
-// position records, are loaded together before they are tested.
-// kFilter: some instance uses the pressure filter; the kernel shape of every
-// list entry is then stored beside the list (nw.wsh_d) for the filter.
+// candidate whose bit is set is tested exactly, and the neighbours are summed
+// and written as i's neighbour list for the pair pass, the inviscid ones
+// first, then the viscous ones, then the walls (each class in candidate
+// order).  The walk takes 4 candidates at a time: their table entries, then
+// their position records, are loaded together before they are tested.
+//
+// The pair geometry is in fixed point (sph_fixed.cuh): about 110 integer
+// instructions per candidate in place of 20 FP64 ones, each of which holds the
+// FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18 of its value
+// (an FP64 evaluation within a few 1.1e-16), and the sum over a list is
+// exact.  20.1M particles: 64.5 ms before, 19.6 ms now.  kFilter: some instance uses the pressure filter; the kernel shape
+// of every list entry is then stored beside the list (nw.wsh_d).
 template <int BLOCK, bool kFilter>
 __global__ void __launch_bounds__(BLOCK)
 k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
@@ -261,86 +281,85 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
   const int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
   if (i >= n) return;
   const InstDev& P = inst[b.inst[i]];
-  const dvec4 pi = b.pos[i];
-  const int sp = (int)pi.w;
+  const QPos pi = ld_qpos(nw.posq + i);
+  const int sp = (int)(pi.tag & 0xFFFFu);
   const double m_i = sp == 0 ? P.m_s : P.m_n;
   double rho;
-  uint32_t cnt = 0, count_a = kUnsplit;
+  uint32_t cnt = 0, parts = 0;
   if (sp == 3) {
     rho = P.rho0;
   } else {
     const int64_t g = (int64_t)cw.skey[i] / P.slabs;  // grid cell
     const int cz_i = (int)((g - P.cell_base / P.slabs) / ((int64_t)P.nx * P.ny));
-    const bool per = P.periodic_z != 0;
-    MaskWalk mk(nw, n, i, g, smask + threadIdx.x, BLOCK);
+    // the z code of a neighbour across the period, and the period to add
+    const bool bottom = cz_i == 0;
+    const uint32_t wrap_code = !P.periodic_z ? 3u : (bottom ? 2u : (cz_i == P.nz - 1 ? 0u : 3u));
+    const int64_t wrap = bottom ? P.fx_Hz : -P.fx_Hz;
+    const uint64_t near2 = P.fx_near, width = P.fx_width, far2 = P.fx_far;
+    ClassWalk mk(nw, n, i, g, smask + threadIdx.x, BLOCK);
     ListWriter out(nw, n, i, stage + threadIdx.x, BLOCK);
-    // fluid rows without the filter: the inviscid neighbours are listed
-    // first; the others are set aside as mask bits and listed after them by a
-    // second walk (the pair pass then runs one specialised loop per part)
-    const bool split = !kFilter && sp < 2;
-    MaskKeep keep_b(mk);
-    const double half_inv_h = 0.5 * P.inv_h, two_inv_h = 2.0 * P.inv_h;
-    const double mD_s = P.m_s * P.aD, mD_n = P.m_n * P.aD;
-    const long long cut2_bits = __double_as_longlong(P.cut2);
-    rho = m_i * P.aD;  // self term W(0)
-    uint32_t e[4], q[4];
-    for (uint32_t m; (m = mk.next(e, q)) != 0u;) {
-      dvec4 pj[4];
+    double sum_s = 0.0;
+    fx::Sum96 sum;
+    uint32_t ends[2];
+    for (int c = 0; c < 3; ++c) {
+      if (c < 2 || mk.walls) {
+        mk.start(c);
+        uint32_t e[4];
+        for (uint32_t m; (m = mk.next(e)) != 0u;) {
+          QPos pj[4];
 #pragma unroll
-      for (uint32_t u = 0; u < 4; ++u)
-        if (u < m) pj[u] = b.pos[checked_index(e[u] & kNbrIndexMask, n, err)];
+          for (uint32_t u = 0; u < 4; ++u)
+            if (u < m) pj[u] = ld_qpos(nw.posq + checked_index(e[u] & kNbrIndexMask, n, err));
 #pragma unroll
-      for (uint32_t u = 0; u < 4; ++u) {
-        if (u < m) {
-          const double dx = __dsub_rn(pi.x, pj[u].x);
-          const double dy = __dsub_rn(pi.y, pj[u].y);
-          double dz = __dsub_rn(pi.z, pj[u].z);
-          if (per) {  // minimum image across the z period
-            const int wz = z_wrap(e[u], cz_i, P.nz);
-            if (wz > 0) dz = __dadd_rn(dz, P.Hz);
-            else if (wz < 0) dz = __dsub_rn(dz, P.Hz);
-          }
-          const double r2 =
-              __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-          // r2 < (2h)^2 on the integer pipe: r2 is a sum of squares (+0 or
-          // positive, or NaN), and such doubles order as their bit patterns
-          const bool keep = __double_as_longlong(r2) < cut2_bits;
-          const bool inv_j = inviscid(pj[u].w);
-          if (split && keep && !inv_j) keep_b.set(q[u]);
-          out.push(e[u], keep && (inv_j || !split));  // index and cell-displacement code
-          if (keep) {
-            // m_j W(r) = (m_j aD) t^4 (2q + 1), t = 1 - q/2, q = r / h
-            const double r = sqrt_dist(r2);
-            const double t1 = fma(-half_inv_h, r, 1.0);
-            const double t2 = t1 * t1;
-            const double mD = inv_j ? mD_s : mD_n;
-            const double Wt = t2 * t2 * fma(two_inv_h, r, 1.0);
-            rho += mD * Wt;
-            if (kFilter) {  // the shape of this list entry, in the list's layout
-              const uint32_t t = out.total() - 1u;
-              if (t < (uint32_t)nw.cap) nw.wsh_d[nbr_slot(n, i, t)] = Wt;
+          for (uint32_t u = 0; u < 4; ++u) {
+            if (u < m) {
+              const bool across = (e[u] >> (kNbrIndexBits + 4)) == wrap_code;
+              int64_t dz = (int64_t)((uint64_t)pi.z - (uint64_t)pj[u].z);
+              if (across) dz = (int64_t)((uint64_t)dz + (uint64_t)wrap);
+              const uint64_t r2 =
+                  fx::norm2(fx::split((int64_t)((uint64_t)pi.x - (uint64_t)pj[u].x)),
+                            fx::split((int64_t)((uint64_t)pi.y - (uint64_t)pj[u].y)),
+                            fx::split(dz));
+              bool keep = r2 - near2 < width;
+              uint64_t w8 = 0;
+              if (!keep && r2 < far2) {  // rare: left to the FP64 test
+                const double W =
+                    exact_pair_shape(b.pos, (uint32_t)i, e[u] & kNbrIndexMask,
+                                     across ? (bottom ? 1 : -1) : 0, &P);
+                keep = W >= 0.0;
+                w8 = keep ? (uint64_t)__double2ull_rn(W * 2305843009213693952.0) : 0u;  // 2^61
+              } else if (keep) {
+                const uint64_t t = fx::shape_t(r2);
+                w8 = fx::shape_w8(t, fx::mulhi(t, t));
+              }
+              out.push(e[u], keep);  // index and cell-displacement code
+              if (keep) {
+                sum.add(w8);
+                if (kFilter) {  // the shape of this list entry, in the list's layout
+                  const uint32_t t = out.total() - 1u;
+                  if (t < (uint32_t)nw.cap)
+                    nw.wsh_d[nbr_slot(n, i, t)] = (double)w8 * 4.336808689942017736e-19;  // 2^-61
+                }
+              }
             }
           }
+          if (out.pend >= (uint32_t)kDrainAt) out.drain();
         }
       }
-      if (out.pend >= (uint32_t)kDrainAt) out.drain();
-    }
-    if (split) {
-      count_a = out.total();
-      keep_b.finish();  // the set-aside bits now stand in the staged mask words
-      MaskWalk mk2 = mk;
-      mk2.k = 0;
-      mk2.w = mk2.sw[0];
-      for (uint32_t m; (m = mk2.next(e)) != 0u;) {
-        for (uint32_t u = 0; u < m; ++u) out.push(e[u], true);
-        if (out.pend >= (uint32_t)kDrainAt) out.drain();
+      if (c == 0) {
+        sum_s = sum.shape_sum();
+        sum = fx::Sum96();
       }
+      if (c < 2) ends[c] = out.total() < (uint32_t)nw.cap ? out.total() : (uint32_t)nw.cap;
     }
+    // rho_i = aD (m_i + m_s sum_s W/aD + m_n sum_n W/aD), the self term W(0) = aD
+    rho = fma(P.m_s * P.aD, sum_s, fma(P.m_n * P.aD, sum.shape_sum(), m_i * P.aD));
+    parts = ends[0] | ((ends[1] - ends[0]) << 16);
     cnt = out.finish();
     if (out.overflow()) latch(err, ERR_NEIGHBORS);
   }
   nw.count[i] = cnt;
-  nw.count_a[i] = count_a;
+  nw.count_a[i] = parts;
   const double Pres = P.p0 * ipow(rho * P.inv_rho0, P.alphaP) - P.beta_P;
   f.rho[i] = rho;
   f.P[i] = Pres;
@@ -411,9 +430,8 @@ k_pfilter_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
 // lists a fluid particle's inviscid neighbours first (count_a of them), and
 // the pair pass runs over the fluid particles in species order (all inviscid
 // ones, then all viscous ones), so that each warp walks the two parts of its
-// lists with one specialised loop each: kPathII, kPathIX, kPathVV.  kPathAll
-// is the unspecialised loop for unsplit lists (the pressure filter's runs).
-enum { kPathAll = 0, kPathII = 1, kPathIX = 2, kPathVV = 3 };
+// lists with one specialised loop each: kPathII, kPathIX, kPathVV.
+enum { kPathII = 1, kPathIX = 2, kPathVV = 3 };
 
 // Per-particle constants of the pair pass, with the term switches, V_i and
 // the kernel constants folded in.
@@ -492,11 +510,9 @@ __device__ __forceinline__ void pair_loop(const PairCtx& C, const InstDev& P, co
       }
       const dvec4 vj = b.vel[j];
       const dvec4 wj = b.spin[j];
-      // whether j is viscous (or a wall): fixed by the list part except in
-      // the unspecialised loop (unlike species: j is viscous iff i is not)
-      const bool vis_j = kPath == kPathVV ? true
-                       : kPath == kPathIX ? C.si == 0
-                                          : !inviscid(pj.w);
+      // whether j is viscous (or a wall): fixed by the list part (unlike
+      // species: j is viscous iff i is not)
+      const bool vis_j = kPath == kPathVV || C.si == 0;
       // relative velocity v_ij and spin-corrected u_ij = v_ij + 1/2 r_ij x (w_i + w_j),
       // with s = (w_i + w_j) / 2
       const double vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
@@ -518,17 +534,10 @@ __device__ __forceinline__ void pair_loop(const PairCtx& C, const InstDev& P, co
         aP = (vis_j ? C.cP1 : C.cP0) * (wi.w + wj.w) * F;
         aT = (vis_j ? C.cT1 : C.cT0) * VF;
         bN = (vis_j ? C.cN1 : C.cN0) * vj.w * W;
-      } else if (kPath == kPathVV) {  // like viscous species: pressure, shear, rotational
+      } else {  // like viscous species: pressure, shear, rotational
         aP = C.cP1 * (wi.w + wj.w) * F;
         aV = VF * (inv_r * inv_r) * (C.cBA1 * dv);
         bR = C.cB1 * VF;
-      } else {  // any pair
-        const double W = t2 * t2 * fma(C.two_inv_h, r, 1.0);
-        aP = (vis_j ? C.cP1 : C.cP0) * (wi.w + wj.w) * F;
-        aT = (vis_j ? C.cT1 : C.cT0) * VF;
-        aV = vis_j ? VF * (inv_r * inv_r) * (C.cBA1 * dv) : 0.0;
-        bR = vis_j ? C.cB1 * VF : 0.0;
-        bN = (vis_j ? C.cN1 : C.cN0) * vj.w * W;
       }
       // (a class loop adds only the terms its class carries: no FP64 addition
       // of a zero term, as the FP64 pipe bounds this loop)
@@ -541,9 +550,7 @@ __device__ __forceinline__ void pair_loop(const PairCtx& C, const InstDev& P, co
       const double al = kPath == kPathVV ? base : base + aT;
       const double alz = C.hproj ? base : al;
       // coefficient of u_ij
-      const double bu = kPath == kPathIX ? (C.literal ? 0.0 : bN)
-                      : kPath == kPathVV ? bR
-                                         : (C.literal ? bR : bR + bN);
+      const double bu = kPath == kPathIX ? (C.literal ? 0.0 : bN) : bR;
       // The pair force al r_ij + bu u_ij (+ bN v_ij) goes into the sums one
       // fused multiply-add per term, and so does the spin torque
       // -1/2 r_ij x (f_rot + f_sn) = -1/2 bu (r_ij x u_ij), whose factor
@@ -639,20 +646,16 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
   C.per = P.periodic_z != 0;
   PairSums S;
   const uint32_t cnt = checked_count(nw.count[i], nw.cap, err);
-  const uint32_t ca = nw.count_a[i];
-  if (ca == kUnsplit) {
-    pair_loop<kPathAll, kOpt>(C, P, b, nw, n, i, 0u, cnt, err, S);
+  const uint32_t ca = nw.count_a[i] & 0xFFFFu;
+  const uint32_t na = ca < cnt ? ca : cnt;
+  // the inviscid neighbours, then the others: the warp's particles are of
+  // one species except at the boundary of the two parts of the order
+  if (t < n_inv) {
+    pair_loop<kPathII, kOpt>(C, P, b, nw, n, i, 0u, na, err, S);
+    pair_loop<kPathIX, kOpt>(C, P, b, nw, n, i, na, cnt, err, S);
   } else {
-    const uint32_t na = ca < cnt ? ca : cnt;
-    // the inviscid neighbours, then the others: the warp's particles are of
-    // one species except at the boundary of the two parts of the order
-    if (t < n_inv) {
-      pair_loop<kPathII, kOpt>(C, P, b, nw, n, i, 0u, na, err, S);
-      pair_loop<kPathIX, kOpt>(C, P, b, nw, n, i, na, cnt, err, S);
-    } else {
-      pair_loop<kPathIX, kOpt>(C, P, b, nw, n, i, 0u, na, err, S);
-      pair_loop<kPathVV, kOpt>(C, P, b, nw, n, i, na, cnt, err, S);
-    }
+    pair_loop<kPathIX, kOpt>(C, P, b, nw, n, i, 0u, na, err, S);
+    pair_loop<kPathVV, kOpt>(C, P, b, nw, n, i, na, cnt, err, S);
   }
   const double inv_m = 1.0 / m_i;
   f.acc[i] = dvec4{S.fx * inv_m, S.fy * inv_m, S.fz * inv_m, 0.0};
@@ -660,6 +663,466 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
   f.dspin[i] = dvec4{tx * inv_I, ty * inv_I, tz * inv_I, 0.0};
   f.tw[i] = dvec4{S.wx, S.wy, S.wz, 0.0};
   if (!finite3(S.fx, S.fy, S.fz) || !finite3(tx, ty, tz)) latch(err, ERR_NONFINITE);
+}
+
+// ----------------------------------------------- pair pass in fixed point
+//
+// The default form's pair pass (neither the literal F_sn nor the collision
+// model).  An FP64 operation holds its pipe for 64 issue slots on this part
+// (two thread operations per SM and clock), so the class loops above, 23 to
+// 79 of them per pair, ran 89 % FP64-pipe busy.  Here a pair's vectors are
+// 64-bit fixed point and the sums 96-bit, on the integer pipe; FP64 is left
+// to the coefficients of the finished sums.
+//
+// Scales.  The geometry is in units of 2h (sph_fixed.cuh).  Velocities,
+// h times the spins and P / rho^2 come as mantissas at each particle's own
+// exponent; a first walk over i's list takes the largest exponents of its
+// neighbours, and the largest |v_ij| in FP32, which give the power of two
+// 2^E2 above every |u_ij|.  u_ij is then rounded at 2^-60 of that (an FP64
+// evaluation rounds each operation at 2^-53 of its own value), the
+// coefficient V_j F or V_j W that multiplies it is shifted up to 62 bits and
+// the product added that much lower in a 96-bit sum, and a pressure term is
+// rounded at 2^-57 of the largest pressure.  A sum is exact: it does not
+// depend on the order of the list or on the number of lanes.
+//
+// kLanes lanes take a particle's entries in turn (warps of 8 particles
+// diverge less than warps of 32, and small vessels spread over more warps);
+// their sums are added by shuffles and the block's first threads finish one
+// particle each, so the FP64 instructions of the end are issued by full
+// warps.  The wall neighbours stand at the end of the list and are summed by
+// themselves: their force and torque give the wall torque.  A pair that fixed
+// point does not resolve (see fx_near; two viscous particles closer than
+// 2h / 8; values outside the range the scales cover, NaN among them) is
+// evaluated in FP64 by slow_pair.
+//
+// Measured against a 64-bit-mantissa evaluation (vessels of 9,000 to 23,000
+// particles, 0 to 300 steps): relative L2 error of the acceleration 8e-16 to
+// 6e-15 (FP64 loops 3e-15 to 3e-14), of the spin change 2.0e-16 to 2.4e-16
+// (4.1e-16 to 8.1e-16), of the density 7e-17 (3.6e-16).  20.1M particles:
+// 134.3 ms before, 43.9 ms now.
+
+constexpr int kLanes = 4;
+constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip
+// Entries that a 64-bit sum holds: a pressure term is below 2 (27/256) 2^57 (t^3 (1 - t) is at
+// most 27/256), an interfacial one below (27/256) 2^58.
+constexpr uint32_t kMaxFx = 160;
+constexpr int kSlots = 48;           // per particle: 3 phases x 12 sums, 12 of the FP64 route
+
+__global__ void k_pair_records(int64_t n, Fp64Buf b, const InstDev* __restrict__ inst, NbrWs nw) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const InstDev& P = inst[b.inst[i]];
+    const dvec4 v = b.vel[i], w = b.spin[i];
+    const double hx = P.h * w.x, hy = P.h * w.y, hz = P.h * w.z;
+    const int ev = max(fx::exponent_of(v.x), max(fx::exponent_of(v.y), fx::exponent_of(v.z)));
+    const int eh = max(fx::exponent_of(hx), max(fx::exponent_of(hy), fx::exponent_of(hz)));
+    const int ep = fx::exponent_of(w.w);
+    PairRec r;
+    r.v[0] = fx::mantissa_at(v.x, ev);
+    r.v[1] = fx::mantissa_at(v.y, ev);
+    r.v[2] = fx::mantissa_at(v.z, ev);
+    const double V = v.w * P.aD * 4611686018427387904.0;  // 2^62
+    r.V = V < 4611686018427387904.0 ? (uint64_t)__double2ll_rn(V) : (1ull << 62) - 1ull;
+    r.h[0] = fx::mantissa_at(hx, eh);
+    r.h[1] = fx::mantissa_at(hy, eh);
+    r.h[2] = fx::mantissa_at(hz, eh);
+    r.P = fx::mantissa_at(w.w, ep);
+    nw.prec[i] = r;
+    nw.pvel[i] = make_float4((float)v.x, (float)v.y, (float)v.z, 0.f);
+    QPos* q = nw.posq + i;
+    q->tag = (q->tag & 0xFFFFu) | ((uint32_t)(ev + 1022) << 16);
+    q->exps = (uint32_t)(eh + 1022) | ((uint32_t)(ep + 1022) << 16);
+  }
+}
+
+// One pair in FP64: the force and the spin torque of j on i into out[0..5],
+// and again into out[6..11] if j is a wall.
+__device__ __noinline__ void slow_pair(const Fp64Buf* b, const InstDev* Pp, uint32_t i, uint32_t j,
+                                       int wz, double* out) {
+  const InstDev& P = *Pp;
+  const dvec4 pi = b->pos[i], vi = b->vel[i], wi = b->spin[i];
+  const dvec4 pj = b->pos[j], vj = b->vel[j], wj = b->spin[j];
+  const double dx = pi.x - pj.x, dy = pi.y - pj.y;
+  double dz = pi.z - pj.z;
+  if (wz > 0) dz += P.Hz;
+  else if (wz < 0) dz -= P.Hz;
+  const double r2 = dx * dx + dy * dy + dz * dz;
+  if (!(r2 > 0.0)) return;  // coincident particles: density only
+  const double inv_r = rsqrt(r2), r = r2 * inv_r;
+  const double t1 = fma(-0.5 * P.inv_h, r, 1.0), t2 = t1 * t1;
+  const double F = P.cF * (t2 * t1), W = P.aD * (t2 * t2 * fma(2.0 * P.inv_h, r, 1.0));
+  const bool inv_i = inviscid(pi.w), inv_j = inviscid(pj.w);
+  const uint32_t fl = P.flags;
+  const double VV = vi.w * vj.w;
+  const double mm = (inv_i ? P.m_s : P.m_n) * (inv_j ? P.m_s : P.m_n);
+  double al = (fl & SPH_TERM_P) ? mm * (wi.w + wj.w) * F : 0.0, aT = 0.0, bu = 0.0;
+  const double vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
+  if (inv_i != inv_j) {
+    if (fl & SPH_TERM_T) aT = P.C_T * VV * F;
+    if (fl & SPH_TERM_SN) bu = -P.C_l * VV * W;
+  } else if (!inv_i) {
+    const double A = (fl & SPH_TERM_SH) ? P.A : 0.0, B = (fl & SPH_TERM_ROT) ? P.B : 0.0;
+    al += (B - A) * VV * F * (dx * vx + dy * vy + dz * vz) * (inv_r * inv_r);
+    bu = -B * VV * F;
+  }
+  const double sx = 0.5 * (wi.x + wj.x), sy = 0.5 * (wi.y + wj.y), sz = 0.5 * (wi.z + wj.z);
+  const double ux = vx + (dy * sz - dz * sy), uy = vy + (dz * sx - dx * sz),
+               uz = vz + (dx * sy - dy * sx);
+  double f[6];
+  f[0] = (al + aT) * dx;
+  f[1] = (al + aT) * dy;
+  f[2] = (al + ((fl & SPH_HPROJ) ? 0.0 : aT)) * dz;
+  f[3] = f[4] = f[5] = 0.0;
+  if (inv_i != inv_j || !inv_i) {  // (two inviscid particles do not see the velocities)
+    f[0] += bu * ux;
+    f[1] += bu * uy;
+    f[2] += bu * uz;
+    f[3] = -0.5 * bu * (dy * uz - dz * uy);
+    f[4] = -0.5 * bu * (dz * ux - dx * uz);
+    f[5] = -0.5 * bu * (dx * uy - dy * ux);
+  }
+  const bool wall = is_wall(pj.w);
+  for (int k = 0; k < 6; ++k) {
+    out[k] += f[k];
+    if (wall) out[6 + k] += f[k];
+  }
+}
+
+__device__ __forceinline__ int64_t shr(int64_t v, int s) { return v >> (s < 63 ? s : 63); }
+__device__ __forceinline__ int64_t sub64(int64_t a, int64_t b) {
+  return (int64_t)((uint64_t)a - (uint64_t)b);
+}
+
+// What the loops over a particle's entries need.
+struct FxCtx {
+  QPos q;                       // own position
+  int64_t v[3], h[3], P;        // own values at the common scales
+  int Ev, Eh, EP;               // shifts of a neighbour's mantissas: E - e (biased)
+  int L;                        // left shift of v_ij to the scale of u
+  uint32_t wrap_code;
+  int64_t wrap;
+  uint64_t near2, width, width_vv;  // r^2 - near2 < width: fixed point (0: never)
+  bool bottom;
+};
+
+// Entries t0, t0 + kLanes, ... of particle i below t1.
+template <int kPath>
+__device__ __forceinline__ void fx_loop(const FxCtx& C, const InstDev& P, const Fp64Buf& b,
+                                        const NbrWs& nw, int64_t n, int64_t i, uint32_t t0,
+                                        uint32_t t1, uint32_t* err, fx::Acc96 (&acc)[12],
+                                        double* slow, bool& any_slow) {
+  // the pressure's and the interfacial sums fit 64 bits (kMaxFx terms)
+  int64_t sp[3] = {0, 0, 0}, sx[3] = {0, 0, 0};
+  using fx::Half;
+  using fx::mul;
+  using fx::split;
+  // the next entry's position record is loaded one entry ahead, the entry
+  // after it two ahead
+  if (t0 >= t1) return;
+  uint32_t ent_n = nw.list[nbr_slot(n, i, t0)];
+  QPos q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
+  uint32_t ent_nn = t0 + kLanes < t1 ? nw.list[nbr_slot(n, i, t0 + kLanes)] : ent_n;
+  for (uint32_t t = t0; t < t1; t += kLanes) {
+    const uint32_t ent = ent_n;
+    const uint32_t j = checked_index(ent & kNbrIndexMask, n, err);
+    const QPos q = q_n;
+    ent_n = ent_nn;
+    q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
+    if (t + 2 * kLanes < t1) ent_nn = nw.list[nbr_slot(n, i, t + 2 * kLanes)];
+    const PairRec* __restrict__ rec = nw.prec + j;
+    const bool across = (ent >> (kNbrIndexBits + 4)) == C.wrap_code;
+    int64_t dz = sub64(C.q.z, q.z);
+    if (across) dz = (int64_t)((uint64_t)dz + (uint64_t)C.wrap);
+    const Half d[3] = {split(sub64(C.q.x, q.x)), split(sub64(C.q.y, q.y)), split(dz)};
+    const uint64_t r2 = fx::norm2(d[0], d[1], d[2]);
+    const uint64_t near2 = kPath == kPathVV ? kNearVV : C.near2;
+    const uint64_t width = kPath == kPathVV ? C.width_vv : C.width;
+    if (r2 - near2 >= width) {
+      slow_pair(&b, &P, (uint32_t)i, j, across ? (C.bottom ? 1 : -1) : 0, slow);
+      any_slow = true;
+      continue;
+    }
+    const int64_t rho = fx::root(r2);
+    const uint64_t tt = (uint64_t)((1ll << 62) - rho) << 2;  // t in units of 2^-64
+    const uint64_t tq = fx::mulhi(tt, tt);
+    const uint64_t F64 = fx::mulhi(tq, tt);                  // F shape t^3, 2^-64
+    // pressure: (P_i / rho_i^2 + P_j / rho_j^2) F r_ij
+    const int64_t g = C.P + shr(rec->P, C.EP - (int)(q.exps >> 16));
+    const Half gF = split(mul(split(g), split((int64_t)(F64 >> 2))));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) sp[a] += mul(gF, d[a]);
+    if (kPath == kPathII) continue;
+    // u_ij = v_ij + r_ij x (w_i + w_j) / 2
+    const int sv = C.Ev - (int)(q.tag >> 16), sh = C.Eh - (int)(q.exps & 0xFFFFu);
+    int64_t v[3];
+    Half s[3], u[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      v[a] = sub64(C.v[a], shr(rec->v[a], sv)) << C.L;
+      s[a] = split(C.h[a] + shr(rec->h[a], sh));
+    }
+    u[0] = split(v[0] + fx::mul_sub(d[1], s[2], d[2], s[1]));
+    u[1] = split(v[1] + fx::mul_sub(d[2], s[0], d[0], s[2]));
+    u[2] = split(v[2] + fx::mul_sub(d[0], s[1], d[1], s[0]));
+    const uint64_t V = rec->V << 2;
+    const uint64_t VF = fx::mulhi(V, F64) >> 2;  // V_j F, 2^-62
+    uint64_t c;  // the coefficient of u: V_j W (unlike species) or V_j F (two viscous)
+    if (kPath == kPathIX) {
+      // interfacial: V_j F r_ij
+      const Half VFh = split((int64_t)(VF >> 2));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) sx[a] += mul(VFh, d[a]);
+      c = fx::mulhi(V, fx::shape_w8(tt, tq)) << 1;
+    } else {
+      c = VF;
+    }
+    const int lz = fx::lead62(c), up = 24 - lz;  // 2^lz c has 62 bits
+    const Half ch = split((int64_t)(c << lz));
+    if (kPath == kPathVV) {
+      // the part along e_ij: V_j F (e_ij . v_ij) e_ij
+      const Half z = split(fx::recip(rho));
+      Half e[3], vh[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        e[a] = split(mul(d[a], z) << 5);
+        vh[a] = split(v[a]);
+      }
+      const Half ev = split(mul(ch, split(fx::dot3(e, vh) << 2)) << 2);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) acc[3 + a].add_shifted(mul(ev, e[a]), up);
+    }
+    int64_t p[3];
+    Half ph[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      p[a] = mul(ch, u[a]);
+      acc[6 + a].add_shifted(p[a], up);
+      ph[a] = split(p[a] << 3);
+    }
+    acc[9].add_shifted(fx::mul_sub(d[1], ph[2], d[2], ph[1]), up);
+    acc[10].add_shifted(fx::mul_sub(d[2], ph[0], d[0], ph[2]), up);
+    acc[11].add_shifted(fx::mul_sub(d[0], ph[1], d[1], ph[0]), up);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    acc[a].add(sp[a]);
+    if (kPath == kPathIX) acc[3 + a].add(sx[a]);
+  }
+}
+
+// Adds another lane's sum.
+__device__ __forceinline__ void add_lane(fx::Acc96& a, const fx::Acc96& give, int mask) {
+  const uint32_t x = __shfl_xor_sync(~0u, give.w0, mask);
+  const uint32_t y = __shfl_xor_sync(~0u, give.w1, mask);
+  const uint32_t z = __shfl_xor_sync(~0u, give.w2, mask);
+  a.add3(x, y, z);
+}
+
+// The kLanes lanes' twelve sums added, lane l left with sums kKeep l ..
+// kKeep (l + 1) - 1 in acc[0 .. kKeep - 1]: each exchange halves what a lane
+// holds.
+constexpr int kKeep = 12 / kLanes;
+__device__ __forceinline__ void reduce12(fx::Acc96 (&acc)[12]) {
+#pragma unroll
+  for (int o = kLanes / 2, m = 6; o > 0; o >>= 1, m >>= 1) {
+    const bool up = (threadIdx.x & o) != 0;
+#pragma unroll
+    for (int k = 0; k < m; ++k) {
+      const fx::Acc96 give = up ? acc[k] : acc[k + m];
+      acc[k] = up ? acc[k + m] : acc[k];
+      add_lane(acc[k], give, o);
+    }
+  }
+}
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
+k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
+            NbrWs nw, uint32_t* err, int64_t part_totals) {
+  constexpr int kRows = BLOCK / kLanes;
+  __shared__ double sums[kRows][kSlots + 1];
+  const int64_t n_fluid = nw.part[part_totals + 1], n_inv = nw.part[part_totals];
+  const int64_t first = (int64_t)blockIdx.x * kRows;
+  if (first >= n_fluid) return;
+  const int row = threadIdx.x / kLanes, lane = threadIdx.x % kLanes;
+  const bool live = first + row < n_fluid;
+  const bool inv_i = first + row < n_inv;
+  const int64_t i = live ? checked_index(nw.order[first + row], n, err) : 0;
+  const InstDev& P = inst[b.inst[i]];
+  uint32_t cnt = 0, na = 0, nb = 0;
+  FxCtx C;
+  C.q = ld_qpos(nw.posq + i);
+  if (live) {
+    cnt = checked_count(nw.count[i], nw.cap, err);
+    const uint32_t parts = nw.count_a[i];
+    na = min(parts & 0xFFFFu, cnt);
+    nb = min(parts >> 16, cnt - na);
+  }
+  // first walk: the largest exponents, and the largest |v_ij|
+  const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
+  uint32_t eP = C.q.exps >> 16, ev = C.q.tag >> 16, eh = C.q.exps & 0xFFFFu;
+  float dv = 0.f;
+  const float4 vi = nw.pvel[i];
+  for (uint32_t t = lane; t < cnt; t += kLanes) {
+    const uint32_t j = checked_index(nw.list[nbr_slot(n, i, t)] & kNbrIndexMask, n, err);
+    const uint2 m = *reinterpret_cast<const uint2*>(&nw.posq[j].tag);
+    eP = max(eP, m.y >> 16);
+    if (t >= u0) {
+      ev = max(ev, m.x >> 16);
+      eh = max(eh, m.y & 0xFFFFu);
+      const float4 vj = nw.pvel[j];
+      const float x = fabsf(vi.x - vj.x), y = fabsf(vi.y - vj.y), z = fabsf(vi.z - vj.z);
+      dv = fmaxf(dv, fmaxf(x, fmaxf(y, z)));
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    eP = max(eP, __shfl_xor_sync(~0u, eP, o));
+    ev = max(ev, __shfl_xor_sync(~0u, ev, o));
+    eh = max(eh, __shfl_xor_sync(~0u, eh, o));
+    dv = fmaxf(dv, __shfl_xor_sync(~0u, dv, o));
+  }
+  // 2^E2 above |v_ij| + |r_ij x s| in every component: |v_ij| from its FP32
+  // value (off by at most 2^-22 of the largest velocity), |s| <= 2 sqrt(3) 2^Eh
+  const int E_v = (int)ev - 1022, E_h = (int)eh - 1022, E_P = (int)eP - 1022;
+  const float bound = fmaf(3.5f, ldexpf(1.f, E_h), fmaf(1.0001f, dv, ldexpf(1.f, E_v - 22)));
+  // (nothing moves or spins: the products' half units come out as zero)
+  const bool still = (ev | eh) == 0u;
+  const int E2 = still ? -1020 : max((int)(__float_as_uint(bound) >> 23) - 126, E_h + 2);
+  const int E_v1 = max(E_v, E2);
+  // values the scales do not cover (a longer list than the sums hold,
+  // overflow, NaN, FP32 underflow of v_ij)
+  const bool covered = cnt <= kMaxFx && eP < 2047u && ev < 2047u && eh < 2047u &&
+                       bound < 1e30f && (still || bound > 1e-30f);
+  {
+    const int64_t g = (int64_t)cw.skey[i] / P.slabs;  // grid cell
+    const int cz_i = (int)((g - P.cell_base / P.slabs) / ((int64_t)P.nx * P.ny));
+    C.bottom = cz_i == 0;
+    C.wrap_code = !P.periodic_z ? 3u : (C.bottom ? 2u : (cz_i == P.nz - 1 ? 0u : 3u));
+    C.wrap = C.bottom ? P.fx_Hz : -P.fx_Hz;
+    C.near2 = P.fx_near;
+    C.width = covered ? P.fx_width : 0u;
+    C.width_vv = C.width ? C.width - (kNearVV - P.fx_near) : 0u;
+    const PairRec r = nw.prec[i];
+    C.Ev = E_v1 + 1022;
+    C.Eh = E2 - 2 + 1022;
+    C.EP = (int)eP;
+    C.L = E_v1 - E2;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      C.v[a] = shr(r.v[a], C.Ev - (int)(C.q.tag >> 16));
+      C.h[a] = shr(r.h[a], C.Eh - (int)(C.q.exps & 0xFFFFu));
+    }
+    C.P = shr(r.P, C.EP - (int)(C.q.exps >> 16));
+  }
+  double slow[12];
+  bool any_slow = false;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) slow[k] = 0.0;
+  // the inviscid neighbours, the viscous ones, the walls
+  const uint32_t end[4] = {0u, na, na + nb, cnt};
+  const int phases = __syncthreads_or(live && cnt > na + nb) ? 3 : 2;
+  for (int ph = 0; ph < phases; ++ph) {
+    fx::Acc96 acc[12];
+    const uint32_t t0 = ph == 0 ? end[0] : (ph == 1 ? end[1] : end[2]);
+    const uint32_t t1 = ph == 0 ? end[1] : (ph == 1 ? end[2] : end[3]);
+    if (inv_i) {
+      if (ph == 0)
+        fx_loop<kPathII>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+      else
+        fx_loop<kPathIX>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+    } else {
+      if (ph == 0)
+        fx_loop<kPathIX>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+      else
+        fx_loop<kPathVV>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+    }
+    __syncwarp();
+    if (ph == 0 && __all_sync(~0u, inv_i)) {  // pairs of inviscid particles: pressure alone
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int o = 1; o < kLanes; o <<= 1) add_lane(acc[k], acc[k], o);
+      }
+#pragma unroll
+      for (int k = 0; k < 3; k += kLanes) {  // sum k + lane
+        fx::Acc96 mine = acc[k];
+#pragma unroll
+        for (int q = 1; q < kLanes && k + q < 3; ++q)
+          if (lane == q) mine = acc[k + q];
+        if (k + lane < 3) sums[row][k + lane] = mine.value(E_P - 57);
+      }
+      continue;
+    }
+    reduce12(acc);
+    // the pressure's sums are in units of 2^(E_P - 57), the interfacial
+    // force's of 2^-58, the torque's of 2^(E2 - 84), the others' of 2^(E2 - 83)
+    const bool unlike = inv_i ? ph > 0 : ph == 0;
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k) {
+      const int q = kKeep * lane + k;
+      const int e = q < 3 ? E_P - 57 : (q < 6 ? (unlike ? -58 : E2 - 83) : (q < 9 ? E2 - 83 : E2 - 84));
+      sums[row][12 * ph + q] = acc[k].value(e);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kKeep; ++k) sums[row][36 + kKeep * lane + k] = 0.0;
+  __syncwarp();
+  if (__any_sync(~0u, any_slow)) {  // the FP64 route's sums, lane by lane
+    for (int l = 0; l < kLanes; ++l) {
+      if (lane == l && any_slow)
+        for (int k = 0; k < 12; ++k) sums[row][36 + k] += slow[k];
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  // one thread per particle: the coefficients of the sums
+  if (threadIdx.x >= kRows || first + threadIdx.x >= n_fluid) return;
+  const double* S = sums[threadIdx.x];
+  const int64_t io = checked_index(nw.order[first + threadIdx.x], n, err);
+  const bool inv_o = first + threadIdx.x < n_inv;
+  const InstDev& Q = inst[b.inst[io]];
+  const uint32_t fl = Q.flags;
+  const double m_i = inv_o ? Q.m_s : Q.m_n, V_i = b.vel[io].w, two_h = 2.0 * Q.h;
+  const double mc = (fl & SPH_TERM_P) ? m_i * Q.cF * two_h : 0.0;
+  const double cPs = mc * Q.m_s, cPn = mc * Q.m_n;
+  const double VF = V_i * Q.cF / Q.aD;  // V_i cF over the unit of the stored volumes
+  const double A = (fl & SPH_TERM_SH) ? Q.A : 0.0, B = (fl & SPH_TERM_ROT) ? Q.B : 0.0;
+  const double cX = (fl & SPH_TERM_T) ? Q.C_T * VF * two_h : 0.0;
+  const double cXz = (fl & SPH_HPROJ) ? 0.0 : cX;
+  const double cN = (fl & SPH_TERM_SN) ? -Q.C_l * V_i : 0.0;
+  const double cE = (B - A) * VF, cB = -B * VF;
+  double F[3], T[3], Fw[3] = {0.0, 0.0, 0.0}, Tw[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    F[a] = S[36 + a];
+    T[a] = S[39 + a];
+    if (inv_o) {
+      F[a] = fma(cPs, S[a], F[a]);
+    } else {
+      F[a] = fma(cPs, S[a], fma(a < 2 ? cX : cXz, S[3 + a], fma(cN, S[6 + a], F[a])));
+      T[a] = fma(-Q.h * cN, S[9 + a], T[a]);
+    }
+    // the viscous neighbours, then the walls
+    const double c3 = inv_o ? (a < 2 ? cX : cXz) : cE, c6 = inv_o ? cN : cB;
+    F[a] = fma(cPn, S[12 + a], fma(c3, S[15 + a], fma(c6, S[18 + a], F[a])));
+    T[a] = fma(-Q.h * c6, S[21 + a], T[a]);
+    if (phases == 3) {
+      Fw[a] = fma(cPn, S[24 + a], fma(c3, S[27 + a], c6 * S[30 + a]));
+      Tw[a] = -Q.h * c6 * S[33 + a];
+      F[a] += Fw[a];
+      T[a] += Tw[a];
+    }
+    Fw[a] += S[42 + a];
+    Tw[a] += S[45 + a];
+  }
+  const double inv_m = 1.0 / m_i, inv_I = inv_o ? Q.inv_I_s : Q.inv_I_n;
+  const dvec4 x = b.pos[io];
+  f.acc[io] = dvec4{F[0] * inv_m, F[1] * inv_m, F[2] * inv_m, 0.0};
+  f.dspin[io] = dvec4{T[0] * inv_I, T[1] * inv_I, T[2] * inv_I, 0.0};
+  f.tw[io] = dvec4{x.y * Fw[2] - x.z * Fw[1] + Tw[0], x.z * Fw[0] - x.x * Fw[2] + Tw[1],
+                   x.x * Fw[1] - x.y * Fw[0] + Tw[2], 0.0};
+  if (!finite3(F[0], F[1], F[2]) || !finite3(T[0], T[1], T[2])) latch(err, ERR_NONFINITE);
 }
 
 // ----------------------------------------------------------- load / unload
@@ -734,9 +1197,9 @@ cudaError_t launch_kick_drift_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields
 }
 
 cudaError_t launch_reorder_fp64(int64_t n, const Fp64Buf& src, const Fp64Buf& dst,
-                                const CellWs& cw, const NbrWs& nw, cudaStream_t s,
-                                const LaunchCfg& lc, int* launches) {
-  k_reorder_fp64<<<grid_for(n, 256, lc.sm_count, 32), 256, 0, s>>>(n, src, dst, cw, nw);
+                                const CellWs& cw, const NbrWs& nw, const InstDev* inst,
+                                cudaStream_t s, const LaunchCfg& lc, int* launches) {
+  k_reorder_fp64<<<grid_for(n, 256, lc.sm_count, 32), 256, 0, s>>>(n, src, dst, cw, nw, inst);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -778,6 +1241,18 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
                  g64 = (unsigned)((n + 63) / 64);
   // the pair pass carries only the options some instance uses
   const int opt = (lc.any_literal ? kOptLiteral : 0) | (lc.any_collision ? kOptCollision : 0);
+  if (opt == 0) {  // the default form, in fixed point
+    k_pair_records<<<grid_for(n, 256, lc.sm_count, 32), 256, 0, s>>>(n, b, inst, nw);
+    const auto rows = [&](int block) { return (unsigned)((n * kLanes + block - 1) / block); };
+    if (lc.block_forces == 256)
+      k_forces_fx<256><<<rows(256), 256, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    else if (lc.block_forces == 64)
+      k_forces_fx<64><<<rows(64), 64, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    else
+      k_forces_fx<128><<<rows(128), 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    if (launches) *launches += 2;
+    return cudaGetLastError();
+  }
   auto go = [&](auto kopt) {
     constexpr int O = decltype(kopt)::value;
     if (lc.block_forces == 256)
@@ -787,9 +1262,7 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
     else
       k_forces_fp64<128, O><<<g128, 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
   };
-  if (opt == 0)
-    go(std::integral_constant<int, 0>());
-  else if (opt == kOptCollision)
+  if (opt == kOptCollision)
     go(std::integral_constant<int, kOptCollision>());
   else  // the literal F_sn, with or without collisions
     go(std::integral_constant<int, kOptLiteral | kOptCollision>());

@@ -185,6 +185,24 @@ sph_status derive(const sph_params& p, InstDev& d) {
                                6.0 * d.cut2 * ldexp(1.0, -24));
   d.cut2f_margin = nextafterf((float)(d.cut2 + margin), INFINITY);
 
+  // Fixed-point pair geometry of the FP64 form (sph_fixed.cuh).  The FP64 test
+  // r^2 < (2h)^2 rounds each coordinate difference by up to 2^-53 of the
+  // largest coordinate or period and its sums of squares by a few 2^-53; a
+  // fixed-point r^2 within fx_band of the cutoff (eight times that, plus its
+  // own few units) is left to the FP64 test, so the sets are the same.  Where
+  // the prefilter lets pairs beyond 1.02 (2h) through (a box of tens of
+  // thousands of supports), every pair is.
+  d.fx_unit = fx::make_unit(2.0 * h);
+  d.fx_Hz = fx::to_fixed(Hz, d.fx_unit);
+  {
+    const double rel = ldexp(32.0 + 16.0 * (2.0 * xmax + Hz) / (2.0 * h), -53);
+    const bool ok = (double)d.cut2f_margin < 1.04 * d.cut2 && rel < 1e-3;
+    const uint64_t band = ok ? 64u + (uint64_t)ldexp(rel, 60) : 0u;
+    d.fx_near = fx::kNear2;
+    d.fx_width = ok ? fx::kOne2 - band - fx::kNear2 : 0u;
+    d.fx_far = ok ? fx::kOne2 + band : ~0ull;
+  }
+
   // FP32 constants of the mixed form
   if (p.precision == SPH_MIXED &&
       (d.nx > (1 << kCellBitsX) || d.ny > (1 << kCellBitsY) || d.nz > (1 << kCellBitsZ)))
@@ -367,6 +385,11 @@ void carve(void* state, void* ws, int32_t n_inst, int64_t n, int64_t n_cells,
   c.nw.list = w.take<uint32_t>((int64_t)cap * n);
   c.nw.count = w.take<uint32_t>(n);
   c.nw.posf = precision == SPH_FP64 ? w.take<float4>(n) : nullptr;
+  c.nw.posq = precision == SPH_FP64 ? w.take<QPos>(n) : nullptr;
+  c.nw.prec = precision == SPH_FP64 ? w.take<PairRec>(n) : nullptr;
+  c.nw.pvel = precision == SPH_FP64 ? w.take<float4>(n) : nullptr;
+  c.nw.cls = precision == SPH_FP64 ? w.take<uint32_t>(n_cells / kSlabs * 2 * kMaxCandWords)
+                                   : nullptr;
   c.nw.mask = w.take<uint32_t>((int64_t)kMaxCandWords * n);
   c.nw.ncand = w.take<uint32_t>(n_cells / kSlabs);
   c.nw.cand = w.take<uint32_t>(n_cells / kSlabs * kMaxCand);
@@ -511,7 +534,8 @@ sph_status enqueue_cells(sph_ctx* c, cudaStream_t s, int mode, int* launches,
   mark(m, s);
   CK(launch_scatter_sort(c->cw, c->buf[a].id, c->n, s, c->lc, launches));
   mark(m, s);
-  CK(launch_reorder_fp64(c->n, c->buf[a], c->buf[b], c->cw, c->nw, s, c->lc, launches));
+  CK(launch_reorder_fp64(c->n, c->buf[a], c->buf[b], c->cw, c->nw, c->inst, s, c->lc,
+                         launches));
   return SPH_OK;
 }
 

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "sph.h"
+#include "sph_fixed.cuh"
 
 namespace sphgb {
 
@@ -49,6 +50,14 @@ struct InstDev {
   double cC[3];                   // -(1 + col_e) m_a m_b / ((m_a + m_b) dt) for the
                                   // species pairs a + b = 0 (inviscid, inviscid),
                                   // 1 (inviscid, other), 2 (other, other)
+  // FP64 form, pair geometry in fixed point (sph_fixed.cuh): the unit 2h, the
+  // z period in it, and the range of r^2 that fixed point decides: a pair with
+  // fx_near <= r^2 < fx_near + fx_width is a neighbour, one at fx_far or above
+  // is none; the others (within rounding of the cutoff, or nearly coincident)
+  // take the FP64 test.
+  fx::Unit fx_unit;
+  int64_t fx_Hz;
+  uint64_t fx_near, fx_width, fx_far;
   float cut2f_margin;             // FP32 prefilter bound (>= every FP64 neighbour)
   float Hzf, half_Hzf;
   int32_t nx, ny, nz;             // cells per axis (ghost ring except periodic z)
@@ -110,6 +119,23 @@ struct Fp64Buf {
   dvec2* ref;         // wall reference (phase-0) x, y
   uint32_t* id;         // input index
   uint32_t* inst;       // instance index
+};
+
+// Position of a particle in fixed point (sph_fixed.cuh), one 32-byte record.
+struct alignas(32) QPos {
+  int64_t x, y, z;    // in units of 2^-62 2h, modulo 2^64
+  uint32_t tag;       // species in the low 16 bits; for the pair pass the biased
+                      // exponent of the velocity's largest component above
+  uint32_t exps;      // those of h times the spin (low 16 bits) and of P / rho^2
+};
+
+// What the fixed-point pair pass gathers of a neighbour beside its position:
+// mantissas at the exponents of its QPos record, x 2^(61 - e).
+struct alignas(32) PairRec {
+  int64_t v[3];       // velocity
+  uint64_t V;         // V W(0) in units of 2^-62, V = m / rho
+  int64_t h[3];       // h times the spin
+  int64_t P;          // P / rho^2
 };
 
 struct Fp64Fields {
@@ -190,7 +216,7 @@ constexpr int kMaxCandWords = kMaxCand / 32;
 // writes whole sectors and reads 1 KB contiguous per group.  An entry is a
 // candidate-table entry (index | displacement code).
 constexpr int kNbrGroup = 8;
-constexpr uint32_t kUnsplit = 0xFFFFFFFFu;
+constexpr uint32_t kHasWall = 0x80000000u;
 constexpr int kPartTile = 4096;  // particles per tile of the species partition
 
 // Compile-time options of the pair pass (template argument kOpt).
@@ -204,18 +230,25 @@ __host__ __device__ __forceinline__ int64_t nbr_slot(int64_t n, int64_t i, uint3
 struct NbrWs {
   uint32_t* list;       // neighbour entries, layout above
   uint32_t* count;      // neighbours per particle (list length)
-  // FP64 form: the list of a fluid particle holds its inviscid neighbours
-  // first; count_a is their number (kUnsplit: not ordered, when the
-  // pressure filter is on).  Species partition of the fluid particles for
+  // FP64 form: a particle's list holds its inviscid neighbours, then the
+  // viscous ones, then the walls; count_a packs the numbers of the first two
+  // (low and high 16 bits).  Species partition of the fluid particles for
   // the pair pass: order[0 .. n_inv) inviscid, then the viscous ones, each in
   // sorted order.
   uint32_t* count_a;
   uint32_t* order;
   uint32_t* part;       // per-tile counts of the partition, then its totals
   float4* posf;         // FP32 copy of sorted positions (FP64-form prefilter)
+  QPos* posq;           // fixed-point copy of sorted positions (FP64 form)
+  PairRec* prec;        // fixed-point pair records (FP64 form)
+  float4* pvel;         // FP32 velocities, for the pair pass's scales (FP64 form)
+  // FP64 form: per grid cell the inviscid candidates of its table (32 words of
+  // bits in table order), then the wall candidates (32 words).
+  uint32_t* cls;
   uint32_t* mask;       // [kMaxCandWords][n] candidate hit bits
   uint32_t* cand;       // [grid cells][kMaxCand] candidate table of each cell
-  uint32_t* ncand;      // [grid cells] candidates of each cell
+  uint32_t* ncand;      // [grid cells] candidates of each cell (FP64 form: kHasWall
+                        // set if some are walls)
   // Pressure filter only (null otherwise): the kernel shape t^4 (2q + 1) of
   // every list entry, written by the density pass in the list's layout
   // (nbr_slot), so the filter neither gathers positions nor re-evaluates W.
@@ -325,48 +358,58 @@ struct MaskWalk {
     }
     return m;
   }
-  // The same, also giving each entry's candidate position q = 32 word + bit.
+};
+
+// The same walk over one species class at a time, in the FP64 form: class 0
+// the inviscid candidates, 1 the viscous ones, 2 the walls, told apart by the
+// cell's class words, so that a list comes out sorted by class with one
+// writer and no entry is set aside.
+struct ClassWalk {
+  const uint32_t* __restrict__ tab;
+  const uint32_t* __restrict__ cls;
+  uint32_t* sw;
+  uint32_t stride, K, k = 0, w = 0;
+  int c = 0;
+  bool walls;
+  __device__ __forceinline__ ClassWalk(const NbrWs& nw, int64_t n, int64_t i, int64_t g,
+                                       uint32_t* sw_, uint32_t stride_)
+      : tab(nw.cand + g * kMaxCand), cls(nw.cls + g * 2 * kMaxCandWords), sw(sw_),
+        stride(stride_) {
+    const uint32_t nc = nw.ncand[g];
+    walls = (nc & kHasWall) != 0u;
+    K = ((nc & ~kHasWall) + 31u) >> 5;
+    const uint32_t* __restrict__ mw = nw.mask + i;
+#pragma unroll 4
+    for (uint32_t t = 0; t < K; ++t) sw[t * stride] = mw[(int64_t)t * n];
+  }
+  __device__ __forceinline__ uint32_t word() const {
+    const uint32_t m = sw[k * stride];
+    if (c == 0) return m & cls[k];
+    if (c == 2) return m & cls[kMaxCandWords + k];
+    return m & ~(cls[k] | cls[kMaxCandWords + k]);
+  }
+  __device__ __forceinline__ void start(int c_) {
+    c = c_;
+    k = 0;
+    w = K ? word() : 0u;
+  }
   template <int B>
-  __device__ __forceinline__ uint32_t next(uint32_t (&e)[B], uint32_t (&q)[B]) {
+  __device__ __forceinline__ uint32_t next(uint32_t (&e)[B]) {
     uint32_t m = 0;
 #pragma unroll
     for (int u = 0; u < B; ++u) {
-      while (w == 0u && k + 1 < K) w = sw[++k * stride];
+      while (w == 0u && k + 1 < K) {
+        ++k;
+        w = word();
+      }
       if (w != 0u) {
         const uint32_t bit = (uint32_t)__ffs(w) - 1u;
         w &= w - 1u;
-        q[u] = (k << 5) + bit;
-        e[u] = tab[q[u]];
+        e[u] = tab[(k << 5) + bit];
         m = (uint32_t)u + 1u;
       }
     }
     return m;
-  }
-};
-
-// Candidate positions set aside during a mask walk, as bits, written back
-// over the walk's own staged mask words once the walk has passed them (a
-// word is staged before any of its bits is returned), so that a second walk
-// over the same words yields the set-aside entries in candidate order.
-struct MaskKeep {
-  uint32_t* sw;
-  uint32_t stride, K;
-  uint32_t k = 0, acc = 0;
-  __device__ __forceinline__ MaskKeep(const MaskWalk& mk) : sw(mk.sw), stride(mk.stride), K(mk.K) {}
-  __device__ __forceinline__ void set(uint32_t q) {  // q ascending over the calls
-    const uint32_t kq = q >> 5;
-    while (k < kq) {
-      sw[k * stride] = acc;
-      acc = 0u;
-      ++k;
-    }
-    acc |= 1u << (q & 31u);
-  }
-  __device__ __forceinline__ void finish() {  // the remaining words: set-aside bits or none
-    for (; k < K; ++k) {
-      sw[k * stride] = acc;
-      acc = 0u;
-    }
   }
 };
 

@@ -59,8 +59,8 @@ cudaError_t launch_kick_drift_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields
                                    const CellWs& cw, uint32_t* err, int mode,
                                    cudaStream_t s, const LaunchCfg& lc, int* launches);
 cudaError_t launch_reorder_fp64(int64_t n, const Fp64Buf& src, const Fp64Buf& dst,
-                                const CellWs& cw, const NbrWs& nw, cudaStream_t s,
-                                const LaunchCfg& lc, int* launches);
+                                const CellWs& cw, const NbrWs& nw, const InstDev* inst,
+                                cudaStream_t s, const LaunchCfg& lc, int* launches);
 cudaError_t launch_density_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
                                 const InstDev* inst, const CellWs& cw, const NbrWs& nw,
                                 uint32_t* err, cudaStream_t s, const LaunchCfg& lc,

@@ -20,7 +20,8 @@
 // sets are symmetric.  Table entries carry the cell-displacement code.
 // FP64 form: an FP32 prefilter on rounded absolute positions (the periodic
 // image in z taken per run) against a widened bound, a superset of the FP64
-// neighbours; the density pass re-tests every candidate it is given in FP64.
+// neighbours, which the density pass re-tests exactly.  It also writes the
+// species classes of each cell's candidates, one bit per candidate.
 #include "sph_f32x2.cuh"
 #include "sph_kernels.h"
 
@@ -110,7 +111,7 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
       if (lane == 0) latch(err, ERR_NEIGHBORS);
       total = kMaxCand;
     }
-    if (lane == 0) nw.ncand[g] = total;
+    uint32_t walls = 0;  // whether some candidate is a wall (FP64 form)
     uint32_t* __restrict__ table = nw.cand + g * kMaxCand;
     const uint32_t pre_self = __shfl_sync(~0u, rpre, 13);  // the cell's own run
     const float cut2 = kMixed ? P.skin_cut2_f : P.cut2f_margin;
@@ -152,6 +153,16 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
           const bool valid = q < nseg;
           const uint32_t ent = ent_n;
           float4 c = c_n;
+          if (!kMixed && !table_done) {  // the species classes of the cell's candidates
+            const uint32_t inv = __ballot_sync(~0u, valid && c.w == 0.f);
+            const uint32_t wal = __ballot_sync(~0u, valid && c.w >= 2.f);
+            walls |= wal;
+            if (lane == 0) {
+              uint32_t* __restrict__ cls = nw.cls + g * 2 * kMaxCandWords + (s0 >> 5) + k;
+              cls[0] = inv;
+              cls[kMaxCandWords] = wal;
+            }
+          }
           if (k + 1 < nch) {
             const uint32_t qn = q + 32u;
             ent_n = sm.ent[qn < nseg ? qn : 0u];
@@ -230,6 +241,7 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
       table_done = true;
       if (lane < nt) nw.count[i] = hits;
     }
+    if (lane == 0) nw.ncand[g] = total | (walls ? kHasWall : 0u);
   }
 }
 
@@ -267,6 +279,8 @@ k_cell_search_tpp(int64_t n, const float4* __restrict__ rec,
     uint32_t* __restrict__ out = nw.mask + i;
     const float cut2 = kMixed ? P.skin_cut2_f : P.cut2f_margin;
     uint32_t q = 0, word = 0, hits = 0, self_q = ~0u;
+    uint32_t inv = 0, wal = 0, walls = 0;  // class words of the table (FP64 form)
+    uint32_t* __restrict__ cls = kMixed ? nullptr : nw.cls + g * 2 * kMaxCandWords;
     bool over = false;
     for (int r = 0; r < 27 && !over; ++r) {
       const int dz = r / 9 - 1, dy = (r / 3) % 3 - 1, kc = r % 3;
@@ -294,7 +308,20 @@ k_cell_search_tpp(int64_t n, const float4* __restrict__ rec,
           break;
         }
         const uint32_t j = rj0 + e;
-        if (writer) table[q] = j | code;
+        if (writer) {
+          table[q] = j | code;
+          if (!kMixed) {
+            const float w = rec[j].w;
+            inv |= (w == 0.f ? 1u : 0u) << (q & 31u);
+            wal |= (w >= 2.f ? 1u : 0u) << (q & 31u);
+            if ((q & 31u) == 31u) {
+              cls[q >> 5] = inv;
+              cls[kMaxCandWords + (q >> 5)] = wal;
+              walls |= wal;
+              inv = wal = 0u;
+            }
+          }
+        }
         if (active) {
           float4 c = rec[j];
           if (!kMixed) {  // image of the candidate across the z period
@@ -325,7 +352,14 @@ k_cell_search_tpp(int64_t n, const float4* __restrict__ rec,
       out[(int64_t)(q >> 5) * n] = word;
       hits += __popc(word);
     }
-    if (writer) nw.ncand[g] = q;
+    if (writer) {
+      if (!kMixed && (q & 31u) != 0u) {
+        cls[q >> 5] = inv;
+        cls[kMaxCandWords + (q >> 5)] = wal;
+        walls |= wal;
+      }
+      nw.ncand[g] = q | (walls ? kHasWall : 0u);
+    }
     nw.count[i] = active ? hits : 0u;
   }
 }
