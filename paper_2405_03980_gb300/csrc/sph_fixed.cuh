@@ -123,7 +123,9 @@ SPH_FX u64 norm2(const Half& x, const Half& y, const Half& z) {
 
 SPH_FX float inv_sqrt(float x) {
 #ifdef __CUDA_ARCH__
-  return rsqrtf(x);
+  float y;  // (x is a normal number: no scaling around the hardware estimate)
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 #else
   return 1.0f / sqrtf(x);
 #endif
@@ -141,8 +143,8 @@ SPH_FX int near_int(float x) {
 
 // sqrt(r2) for kNear2 <= r2 < 2^60, in units of 2^-32: an integer estimate r0
 // from the FP32 reciprocal square root y (30 bits, good to about 2^-21), and
-// three corrections e y / 2 of the exact integer residual e = r2 - r^2, which
-// settle the integer part, the next 21 bits and the last 11.
+// two corrections e y / 2 of the exact integer residual e = r2 - r^2, the
+// first down to 2^-12, the second to 2^-32.
 SPH_FX i64 root(u64 r2) {
 #ifdef __CUDA_ARCH__
   const float f = __uint2float_rn((uint32_t)(r2 >> 28));
@@ -150,19 +152,17 @@ SPH_FX i64 root(u64 r2) {
   const float f = (float)(uint32_t)(r2 >> 28);
 #endif
   const float y = inv_sqrt(f);
-  const float yh = y * 3.0517578125e-05f;  // 1 / (2 r0), 2^-15 y
 #ifdef __CUDA_ARCH__
   const uint32_t r0 = __float2uint_rn(f * y * 16384.0f);
 #else
   const uint32_t r0 = (uint32_t)llrintf(f * y * 16384.0f);
 #endif
+  // 1 / (2 r0) = 2^-15 y
   const i64 e0 = (i64)(r2 - (u64)r0 * r0);
-  const uint32_t r1 = r0 + (uint32_t)near_int((float)(int)(e0 >> 9) * (yh * 512.0f));
-  const int e1 = (int)(r2 - (u64)r1 * r1);
-  const int d = near_int((float)e1 * (yh * 2097152.0f));  // 2^21
-  const i64 e2 = ((i64)e1 << 21) - (((i64)d * (int)r1) << 1) - (((i64)d * d) >> 21);
-  const int d3 = near_int((float)(int)(e2 >> 1) * (yh * 4096.0f));  // 2^11, and the halving
-  return ((i64)r1 << 32) + ((i64)d << 11) + d3;
+  const int d1 = near_int((float)(int)(e0 >> 9) * (y * 64.0f));  // 2^9 2^-15 2^12
+  const i64 e1 = (e0 << 12) - (((i64)d1 * (int)r0) << 1) - (((i64)d1 * d1) >> 12);
+  const int d2 = near_int((float)(int)(e1 >> 1) * (y * 64.0f));  // 2 2^-15 2^20
+  return ((i64)r0 << 32) + ((i64)d1 << 20) + d2;
 }
 
 // t = 1 - r / 2h in units of 2^-64 (r2 as for root: 0 < t < 1).

@@ -41,7 +41,7 @@ __device__ __forceinline__ bool finite3(double a, double b, double c) {
 // non-finite coordinate) is clamped into it and ERR_ESCAPED is latched, so
 // every later access stays inside the cell arrays.
 __device__ __forceinline__ uint32_t cell_key(const InstDev& P, double x, double y, double z,
-                                             uint32_t* err) {
+                                             int sp, uint32_t* err) {
   int c[3];
   const double r[3] = {x, y, z};
   bool bad = false;
@@ -61,12 +61,13 @@ __device__ __forceinline__ uint32_t cell_key(const InstDev& P, double x, double 
     }
   }
   if (bad) latch(err, ERR_ESCAPED);
-  // x-slab of the particle inside its cell
-  int slab = (int)floor(((r[0] - P.lo[0]) * P.inv_cell[0] - (double)c[0]) * P.slabs);
-  slab = slab < 0 ? 0 : (slab >= P.slabs ? P.slabs - 1 : slab);
+  // parts of a cell: the inviscid particles in two x-slabs (short runs for the
+  // sort inside a part), the viscous ones, the walls
+  int part = sp < 2 ? 2 : 3;
+  if (sp == 0) part = (r[0] - P.lo[0]) * P.inv_cell[0] - (double)c[0] < 0.5 ? 0 : 1;
   return (uint32_t)(P.cell_base +
                     ((int64_t)c[0] + (int64_t)P.nx * (c[1] + (int64_t)P.ny * c[2])) * P.slabs +
-                    slab);
+                    part);
 }
 
 inline int grid_for(int64_t n, int threads, int sm_count, int per_sm) {
@@ -132,7 +133,7 @@ __global__ void k_kick_drift_fp64(int64_t n, Fp64Buf b, Fp64Fields f,
       b.vel[i] = v;
       b.spin[i] = w;
     }
-    const uint32_t key = cell_key(P, p.x, p.y, p.z, err);
+    const uint32_t key = cell_key(P, p.x, p.y, p.z, sp, err);
     cw.key[i] = key;
     cw.slot[i] = atomicAdd(&cw.count[key], 1u);
   }
@@ -219,30 +220,15 @@ __device__ __forceinline__ int z_wrap(uint32_t ent, int cz_i, int nz) {
   return (cz_i == 0 && cz == 2u) ? 1 : ((cz_i == nz - 1 && cz == 0u) ? -1 : 0);
 }
 
+// Lanes that share a particle's list in the density pass.
+constexpr int kLanes = 4;
+
 // -------------------------------------------------------------------- density
 
 __device__ __forceinline__ double ipow(double x, int e) {
   double r = 1.0;
   for (int t = 0; t < e; ++t) r *= x;
   return r;
-}
-
-// The FP64 route of a candidate pair whose fixed-point r^2 does not decide it
-// (within rounding of the cutoff, or nearly coincident): the exact test
-// r^2 < (2h)^2 without fused multiply-adds, strict <, and the W shape
-// t^4 (2q + 1) of a neighbour; -1 for a pair outside.
-__device__ __noinline__ double exact_pair_shape(const dvec4* pos, uint32_t i, uint32_t j, int wz,
-                                                const InstDev* P) {
-  const dvec4 a = pos[i], b = pos[j];
-  const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
-  double dz = __dsub_rn(a.z, b.z);
-  if (wz > 0) dz = __dadd_rn(dz, P->Hz);
-  else if (wz < 0) dz = __dsub_rn(dz, P->Hz);
-  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-  if (!(r2 < P->cut2)) return -1.0;
-  const double r = sqrt(r2);
-  const double t1 = fma(-0.5 * P->inv_h, r, 1.0), t2 = t1 * t1;
-  return t2 * t2 * fma(2.0 * P->inv_h, r, 1.0);
 }
 
 // A QPos record in one 256-bit load.
@@ -258,115 +244,278 @@ __device__ __forceinline__ QPos ld_qpos(const QPos* q) {
   return r;
 }
 
-// Density and Tait pressure (Eq. 4), one thread per particle, from the hit
-// bits of the FP32 prefilter of the neighbour search (sph_search.cu): every
-// candidate whose bit is set is tested exactly, and the neighbours are summed
-// and written as i's neighbour list for the pair pass, the inviscid ones
-// first, then the viscous ones, then the walls (each class in candidate
-// order).  The walk takes 4 candidates at a time: their table entries, then
-// their position records, are loaded together before they are tested.
+// What decides a pair in fixed point, and the z code and period of a
+// neighbour across the periodic boundary, for particle i in z cell cz.
+struct PairRange {
+  uint64_t near2, width, far2;  // r^2 - near2 < width: neighbour; r^2 >= far2: not
+  uint32_t wrap_code;
+  int64_t wrap;
+  bool bottom;
+};
+__device__ __forceinline__ PairRange pair_range(const InstDev& P, int cz) {
+  PairRange R;
+  R.near2 = P.fx_near;
+  R.width = P.fx_width;
+  R.far2 = P.fx_far;
+  R.bottom = cz == 0;
+  R.wrap_code = !P.periodic_z ? 3u : (R.bottom ? 2u : (cz == P.nz - 1 ? 0u : 3u));
+  R.wrap = R.bottom ? P.fx_Hz : -P.fx_Hz;
+  return R;
+}
+__device__ __forceinline__ int z_cell(const InstDev& P, uint32_t skey) {
+  const int64_t g = (int64_t)skey / P.slabs;  // grid cell
+  return (int)((g - P.cell_base / P.slabs) / ((int64_t)P.nx * P.ny));
+}
+// The pair vector of particle q and neighbour o by entry ent, in halves.
+struct PairVec {
+  fx::Half d[3];
+  bool across;
+};
+__device__ __forceinline__ PairVec pair_vec(const QPos& q, const QPos& o, uint32_t ent,
+                                            const PairRange& R) {
+  PairVec v;
+  v.across = (ent >> (kNbrIndexBits + 4)) == R.wrap_code;
+  uint64_t dz = (uint64_t)q.z - (uint64_t)o.z;
+  if (v.across) dz += (uint64_t)R.wrap;
+  v.d[0] = fx::split((int64_t)((uint64_t)q.x - (uint64_t)o.x));
+  v.d[1] = fx::split((int64_t)((uint64_t)q.y - (uint64_t)o.y));
+  v.d[2] = fx::split((int64_t)dz);
+  return v;
+}
+
+// The exact test of a pair, r^2 < (2h)^2 without fused multiply-adds, strict
+// <, in FP64; across: the pair meets across the z period.
+__device__ __forceinline__ double exact_r2(const dvec4& a, const dvec4& b, bool across,
+                                           const PairRange& R, const InstDev& P) {
+  const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
+  double dz = __dsub_rn(a.z, b.z);
+  if (across) dz = R.bottom ? __dadd_rn(dz, P.Hz) : __dsub_rn(dz, P.Hz);
+  return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+// The list of a particle whose prefiltered neighbours exceed the list's
+// capacity, by one lane with the exact test: returns their number (those past
+// the capacity are dropped) and the entries of the first two classes.
+__device__ __noinline__ uint32_t exact_list(int64_t n, int64_t i, uint32_t K, uint32_t end0,
+                                            uint32_t end1, const uint32_t* tab, const dvec4* pos,
+                                            const InstDev* P, const NbrWs* nw, const PairRange* R,
+                                            uint32_t* parts) {
+  uint32_t have = 0, c0 = 0, c1 = 0;
+  const dvec4 a = pos[i];
+  for (uint32_t k = 0; k < K; ++k)
+    for (uint32_t m = nw->mask[(int64_t)k * n + i]; m; m &= m - 1u) {
+      const uint32_t q = (k << 5) + (uint32_t)__ffs(m) - 1u, ent = tab[q];
+      const bool across = (ent >> (kNbrIndexBits + 4)) == R->wrap_code;
+      if (!(exact_r2(a, pos[ent & kNbrIndexMask], across, *R, *P) < P->cut2)) continue;
+      if (have < (uint32_t)nw->cap) {
+        nw->list[nbr_slot(n, i, have)] = ent;
+        c0 += q < end0 ? 1u : 0u;
+        c1 += q < end1 ? 1u : 0u;
+      }
+      ++have;
+    }
+  *parts = c0 | ((c1 - c0) << 11);
+  return have;
+}
+
+// The FP64 route of the candidate pairs that fixed point does not decide
+// (within rounding of the cutoff, or nearly coincident), after the common
+// loop has passed over them: the exact test and the W shape t^4 (2q + 1).  A
+// pair beyond 2h gets an entry that names i itself.
+template <bool kFilter>
+__device__ __noinline__ void density_exact(int64_t n, int64_t i, uint32_t t0, uint32_t na,
+                                           uint32_t cnt, const dvec4* pos, const InstDev* Pp,
+                                           const NbrWs* nwp, const PairRange* Rp, fx::Sum96* sums,
+                                           uint32_t* dead) {
+  const InstDev& P = *Pp;
+  const NbrWs& nw = *nwp;
+  const QPos pi = nw.posq[i];
+  for (uint32_t t = t0; t < cnt; t += kLanes) {
+    const int64_t at = nbr_slot(n, i, t);
+    const uint32_t ent = nw.list[at], j = ent & kNbrIndexMask;
+    if ((int64_t)j == i) continue;  // found beyond 2h before
+    const PairVec v = pair_vec(pi, nw.posq[j], ent, *Rp);
+    const uint64_t r2q = fx::norm2(v.d[0], v.d[1], v.d[2]);
+    if (r2q - Rp->near2 < Rp->width || r2q >= Rp->far2) continue;
+    const double r2 = exact_r2(pos[i], pos[j], v.across, *Rp, P);
+    double W = 0.0;
+    if (r2 < P.cut2) {
+      const double t1 = fma(-0.5 * P.inv_h, sqrt(r2), 1.0), t2 = t1 * t1;
+      W = t2 * t2 * fma(2.0 * P.inv_h, sqrt(r2), 1.0);
+      sums[t < na ? 0 : 1].add(__double2ull_rn(W * 2305843009213693952.0));  // 2^61
+    } else {
+      nw.list[at] = (uint32_t)i | (21u << kNbrIndexBits);
+      ++*dead;
+    }
+    if (kFilter) nw.wsh_d[at] = W;
+  }
+}
+
+// Density and Tait pressure (Eq. 4).  kLanes lanes first turn the particle's
+// candidate mask (the search's FP32 prefilter; words dealt out to the lanes)
+// into its list, inviscid neighbours, then viscous ones, then walls, in shared
+// memory; then they walk the list, test every entry, sum the neighbours' W
+// shapes and write it out for the pair pass; one thread per particle forms rho
+// and P.  An entry beyond 2h is replaced by one that names i itself, which the
+// pair pass and the read-outs skip.  (With the bits walked and the pairs
+// evaluated in one loop, a thread per particle, 22 of 32 lanes were active.)
 //
-// The pair geometry is in fixed point (sph_fixed.cuh): about 110 integer
-// instructions per candidate in place of 20 FP64 ones, each of which holds the
+// The pair geometry is in fixed point (sph_fixed.cuh): about 120 integer
+// instructions per entry in place of 20 FP64 ones, each of which holds the
 // FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18 of its value
 // (an FP64 evaluation within a few 1.1e-16), and the sum over a list is
-// exact.  20.1M particles: 64.5 ms before, 19.6 ms now.  kFilter: some instance uses the pressure filter; the kernel shape
-// of every list entry is then stored beside the list (nw.wsh_d).
+// exact.  20.1M particles: 64.5 ms with FP64 arithmetic, 19.6 ms in fixed
+// point with a thread per particle, 14.5 ms now (bound by issue, 68 %, and the
+// ALU).  Lists written by the search instead took 10.5 ms here but 7.2 ms more
+// there.  kFilter: some instance uses the pressure filter; the kernel shape of
+// every list entry is then stored beside the list (nw.wsh_d).
+constexpr uint32_t kStaged = 168;  // entries of a list staged in shared memory; a longer one is
+                                   // written out and read back
 template <int BLOCK, bool kFilter>
 __global__ void __launch_bounds__(BLOCK)
 k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
                NbrWs nw, uint32_t* err) {
-  __shared__ uint32_t smask[BLOCK * kMaxCandWords];
-  __shared__ uint32_t stage[BLOCK * kStageWords];
-  const int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (i >= n) return;
+  constexpr int kRows = BLOCK / kLanes;
+  __shared__ uint32_t staged[kRows][kStaged + 1];
+  __shared__ double sums[kRows][2];
+  __shared__ uint32_t gone[kRows];
+  const int64_t first = (int64_t)blockIdx.x * kRows;
+  const int row = threadIdx.x / kLanes, lane = threadIdx.x % kLanes;
+  const bool live = first + row < n;
+  const int64_t i = live ? first + row : n - 1;
   const InstDev& P = inst[b.inst[i]];
   const QPos pi = ld_qpos(nw.posq + i);
-  const int sp = (int)(pi.tag & 0xFFFFu);
-  const double m_i = sp == 0 ? P.m_s : P.m_n;
-  double rho;
-  uint32_t cnt = 0, parts = 0;
-  if (sp == 3) {
-    rho = P.rho0;
-  } else {
-    const int64_t g = (int64_t)cw.skey[i] / P.slabs;  // grid cell
-    const int cz_i = (int)((g - P.cell_base / P.slabs) / ((int64_t)P.nx * P.ny));
-    // the z code of a neighbour across the period, and the period to add
-    const bool bottom = cz_i == 0;
-    const uint32_t wrap_code = !P.periodic_z ? 3u : (bottom ? 2u : (cz_i == P.nz - 1 ? 0u : 3u));
-    const int64_t wrap = bottom ? P.fx_Hz : -P.fx_Hz;
-    const uint64_t near2 = P.fx_near, width = P.fx_width, far2 = P.fx_far;
-    ClassWalk mk(nw, n, i, g, smask + threadIdx.x, BLOCK);
-    ListWriter out(nw, n, i, stage + threadIdx.x, BLOCK);
-    double sum_s = 0.0;
-    fx::Sum96 sum;
-    uint32_t ends[2];
-    for (int c = 0; c < 3; ++c) {
-      if (c < 2 || mk.walls) {
-        mk.start(c);
-        uint32_t e[4];
-        for (uint32_t m; (m = mk.next(e)) != 0u;) {
-          QPos pj[4];
+  const int64_t g = (int64_t)cw.skey[i] / P.slabs;  // grid cell
+  PairRange R = pair_range(P, z_cell(P, cw.skey[i]));
+  // ---- the list: word k of the mask by lane k % kLanes
+  const bool lists = live && (pi.tag & 0xFFFFu) != 3u;  // outer-wall particles keep none
+  const uint32_t K = lists ? (nw.ncand[2 * g] + 31u) >> 5 : 0u;
+  const uint32_t ends = lists ? nw.ncand[2 * g + 1] : 0u, end0 = ends & 0xFFFFu, end1 = ends >> 16;
+  const uint32_t* __restrict__ tab = nw.cand + g * kMaxCand;
+  uint32_t cnt = 0, part0 = 0, part1 = 0;
+  const uint32_t rounds = __reduce_max_sync(~0u, (K + kLanes - 1) / kLanes);
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t k = r * kLanes + (uint32_t)lane;
+    uint32_t m = k < K ? nw.mask[(int64_t)k * n + i] : 0u;
+    uint32_t incl = (uint32_t)__popc(m);  // inclusive scan over the lanes
+    const uint32_t own = incl;
 #pragma unroll
-          for (uint32_t u = 0; u < 4; ++u)
-            if (u < m) pj[u] = ld_qpos(nw.posq + checked_index(e[u] & kNbrIndexMask, n, err));
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u) {
-            if (u < m) {
-              const bool across = (e[u] >> (kNbrIndexBits + 4)) == wrap_code;
-              int64_t dz = (int64_t)((uint64_t)pi.z - (uint64_t)pj[u].z);
-              if (across) dz = (int64_t)((uint64_t)dz + (uint64_t)wrap);
-              const uint64_t r2 =
-                  fx::norm2(fx::split((int64_t)((uint64_t)pi.x - (uint64_t)pj[u].x)),
-                            fx::split((int64_t)((uint64_t)pi.y - (uint64_t)pj[u].y)),
-                            fx::split(dz));
-              bool keep = r2 - near2 < width;
-              uint64_t w8 = 0;
-              if (!keep && r2 < far2) {  // rare: left to the FP64 test
-                const double W =
-                    exact_pair_shape(b.pos, (uint32_t)i, e[u] & kNbrIndexMask,
-                                     across ? (bottom ? 1 : -1) : 0, &P);
-                keep = W >= 0.0;
-                w8 = keep ? (uint64_t)__double2ull_rn(W * 2305843009213693952.0) : 0u;  // 2^61
-              } else if (keep) {
-                const uint64_t t = fx::shape_t(r2);
-                w8 = fx::shape_w8(t, fx::mulhi(t, t));
-              }
-              out.push(e[u], keep);  // index and cell-displacement code
-              if (keep) {
-                sum.add(w8);
-                if (kFilter) {  // the shape of this list entry, in the list's layout
-                  const uint32_t t = out.total() - 1u;
-                  if (t < (uint32_t)nw.cap)
-                    nw.wsh_d[nbr_slot(n, i, t)] = (double)w8 * 4.336808689942017736e-19;  // 2^-61
-                }
-              }
-            }
-          }
-          if (out.pend >= (uint32_t)kDrainAt) out.drain();
-        }
-      }
-      if (c == 0) {
-        sum_s = sum.shape_sum();
-        sum = fx::Sum96();
-      }
-      if (c < 2) ends[c] = out.total() < (uint32_t)nw.cap ? out.total() : (uint32_t)nw.cap;
+    for (int o = 1; o < kLanes; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(~0u, incl, o, kLanes);
+      if (lane >= o) incl += v;
     }
-    // rho_i = aD (m_i + m_s sum_s W/aD + m_n sum_n W/aD), the self term W(0) = aD
-    rho = fma(P.m_s * P.aD, sum_s, fma(P.m_n * P.aD, sum.shape_sum(), m_i * P.aD));
-    parts = ends[0] | ((ends[1] - ends[0]) << 16);
-    cnt = out.finish();
-    if (out.overflow()) latch(err, ERR_NEIGHBORS);
+    uint32_t at = cnt + incl - own;
+    cnt += __shfl_sync(~0u, incl, kLanes - 1, kLanes);
+    // the bits of the first two classes (positions before their ends)
+    const uint32_t q0 = k << 5;
+    const uint32_t d0 = end0 > q0 ? end0 - q0 : 0u, d1 = end1 > q0 ? end1 - q0 : 0u;
+    part0 += (uint32_t)__popc(d0 >= 32u ? m : m & ((1u << d0) - 1u));
+    part1 += (uint32_t)__popc(d1 >= 32u ? m : m & ((1u << d1) - 1u));
+    for (; m; m &= m - 1u, ++at) {
+      const uint32_t ent = tab[q0 + (uint32_t)__ffs(m) - 1u];
+      if (at < kStaged) staged[row][at] = ent;
+      if (cnt > kStaged && at < (uint32_t)nw.cap) nw.list[nbr_slot(n, i, at)] = ent;
+    }
   }
-  nw.count[i] = cnt;
-  nw.count_a[i] = parts;
-  const double Pres = P.p0 * ipow(rho * P.inv_rho0, P.alphaP) - P.beta_P;
-  f.rho[i] = rho;
-  f.P[i] = Pres;
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    part0 += __shfl_xor_sync(~0u, part0, o);
+    part1 += __shfl_xor_sync(~0u, part1, o);
+  }
+  uint32_t parts = part0 | ((part1 - part0) << 11);
+  bool in_memory = cnt > kStaged;  // the list, past the staging
+  __syncwarp();
+  if (in_memory) {  // rounds before the staging filled up wrote to it alone
+    for (uint32_t t = (uint32_t)lane; t < kStaged && t < (uint32_t)nw.cap; t += kLanes)
+      nw.list[nbr_slot(n, i, t)] = staged[row][t];
+  }
+  if (cnt > (uint32_t)nw.cap) {
+    uint32_t have = 0;
+    if (lane == 0) {
+      have = exact_list(n, i, K, end0, end1, tab, b.pos, &P, &nw, &R, &parts);
+      if (have > (uint32_t)nw.cap) latch(err, ERR_NEIGHBORS);
+    }
+    const uint32_t group = ((1u << kLanes) - 1u) << (threadIdx.x & 31 & ~(kLanes - 1));
+    cnt = min(__shfl_sync(group, have, 0, kLanes), (uint32_t)nw.cap);
+    parts = __shfl_sync(group, parts, 0, kLanes);
+    in_memory = true;
+  }
+  __syncwarp();
+  if (live && lane == 0) nw.count[i] = cnt;
+  // ---- the sum
+  const uint32_t na = part_inv(parts);
+  fx::Sum96 sum[2];  // the inviscid neighbours, the others
+  uint32_t dead = 0;
+  bool undecided = false;
+  const auto entry = [&](uint32_t t) {
+    return in_memory ? nw.list[nbr_slot(n, i, t)] : staged[row][t];
+  };
+  if (lane < (int)cnt) {
+    uint32_t ent_n = entry((uint32_t)lane);  // the next record is loaded one entry ahead
+    QPos q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
+    for (uint32_t t = (uint32_t)lane; t < cnt; t += kLanes) {
+      uint32_t ent = ent_n;
+      const QPos q = q_n;
+      if (t + kLanes < cnt) {
+        ent_n = entry(t + kLanes);
+        q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
+      }
+      const PairVec v = pair_vec(pi, q, ent, R);
+      const uint64_t r2 = fx::norm2(v.d[0], v.d[1], v.d[2]);
+      uint64_t w8 = 0;
+      if (r2 - R.near2 < R.width) {
+        const uint64_t tt = fx::shape_t(r2);
+        w8 = fx::shape_w8(tt, fx::mulhi(tt, tt));
+        if (t < na) sum[0].add(w8);
+        else sum[1].add(w8);
+      } else if (r2 >= R.far2) {
+        ent = (uint32_t)i | (21u << kNbrIndexBits);
+        ++dead;
+      } else {
+        undecided = true;
+      }
+      const int64_t at = nbr_slot(n, i, t);
+      nw.list[at] = ent;
+      if (kFilter) nw.wsh_d[at] = (double)w8 * 4.336808689942017736e-19;  // 2^-61
+    }
+    if (undecided)
+      density_exact<kFilter>(n, i, (uint32_t)lane, na, cnt, b.pos, &P, &nw, &R, sum, &dead);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    dead += __shfl_xor_sync(~0u, dead, o);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t x = __shfl_xor_sync(~0u, sum[k].w0, o), y = __shfl_xor_sync(~0u, sum[k].w1, o),
+                     z = __shfl_xor_sync(~0u, sum[k].w2, o);
+      sum[k].add((uint64_t)y << 32 | x);
+      sum[k].w2 += z;
+    }
+  }
+  if (lane < 2) sums[row][lane] = lane == 0 ? sum[0].shape_sum() : sum[1].shape_sum();
+  if (lane == 0) gone[row] = parts | (min(dead, 1023u) << 22);
+  __syncthreads();
+  // ---- rho and P, one thread per particle
+  const int64_t io = first + threadIdx.x;
+  if (threadIdx.x >= kRows || io >= n) return;
+  const InstDev& Q = inst[b.inst[io]];
+  const int sp = (int)(nw.posq[io].tag & 0xFFFFu);
+  const double m_i = sp == 0 ? Q.m_s : Q.m_n;
+  // rho_i = aD (m_i + m_s sum_s W/aD + m_n sum_n W/aD), the self term W(0) = aD;
+  // outer walls keep rho0
+  double rho = Q.rho0;
+  if (sp != 3)
+    rho = fma(Q.m_s * Q.aD, sums[threadIdx.x][0],
+              fma(Q.m_n * Q.aD, sums[threadIdx.x][1], m_i * Q.aD));
+  nw.parts[io] = gone[threadIdx.x];
+  const double Pres = Q.p0 * ipow(rho * Q.inv_rho0, Q.alphaP) - Q.beta_P;
+  f.rho[io] = rho;
+  f.P[io] = Pres;
   const double V = m_i / rho;
-  b.vel[i].w = V;
-  b.spin[i].w = Pres / (rho * rho);
-  if (P.flags & SPH_PFILTER) f.vp[i] = sp == 3 ? dvec2{0.0, 0.0} : dvec2{V, V * Pres};
+  b.vel[io].w = V;
+  b.spin[io].w = Pres / (rho * rho);
+  if (Q.flags & SPH_PFILTER) f.vp[io] = sp == 3 ? dvec2{0.0, 0.0} : dvec2{V, V * Pres};
   if (!isfinite(rho) || !isfinite(Pres)) latch(err, ERR_NONFINITE);
 }
 
@@ -646,7 +795,7 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
   C.per = P.periodic_z != 0;
   PairSums S;
   const uint32_t cnt = checked_count(nw.count[i], nw.cap, err);
-  const uint32_t ca = nw.count_a[i] & 0xFFFFu;
+  const uint32_t ca = part_inv(nw.parts[i]);
   const uint32_t na = ca < cnt ? ca : cnt;
   // the inviscid neighbours, then the others: the warp's particles are of
   // one species except at the boundary of the two parts of the order
@@ -685,23 +834,26 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // rounded at 2^-57 of the largest pressure.  A sum is exact: it does not
 // depend on the order of the list or on the number of lanes.
 //
-// kLanes lanes take a particle's entries in turn (warps of 8 particles
-// diverge less than warps of 32, and small vessels spread over more warps);
-// their sums are added by shuffles and the block's first threads finish one
+// kL lanes take a particle's entries in turn, two or four of them (warps of 16
+// or 8 particles diverge less than warps of 32, and small vessels spread over
+// more warps; see kPairLanes4); their sums are added by shuffles and the block's first threads finish one
 // particle each, so the FP64 instructions of the end are issued by full
 // warps.  The wall neighbours stand at the end of the list and are summed by
 // themselves: their force and torque give the wall torque.  A pair that fixed
 // point does not resolve (see fx_near; two viscous particles closer than
 // 2h / 8; values outside the range the scales cover, NaN among them) is
-// evaluated in FP64 by slow_pair.
+// evaluated in FP64 by slow_walk.
 //
 // Measured against a 64-bit-mantissa evaluation (vessels of 9,000 to 23,000
 // particles, 0 to 300 steps): relative L2 error of the acceleration 8e-16 to
 // 6e-15 (FP64 loops 3e-15 to 3e-14), of the spin change 2.0e-16 to 2.4e-16
 // (4.1e-16 to 8.1e-16), of the density 7e-17 (3.6e-16).  20.1M particles:
-// 134.3 ms before, 43.9 ms now.
+// 134.3 ms before, 38.6 ms now.
 
-constexpr int kLanes = 4;
+// Particles below which four lanes take a list, else two: four fill the GPU
+// sooner, two spend less on adding up (pair pass with 4 / 2 lanes: 8,960
+// particles 78 / 122 us, 2.5M 5.23 / 4.80 ms).
+constexpr int64_t kPairLanes4 = 1 << 18;
 constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip
 // Entries that a 64-bit sum holds: a pressure term is below 2 (27/256) 2^57 (t^3 (1 - t) is at
 // most 27/256), an interfacial one below (27/256) 2^58.
@@ -799,46 +951,54 @@ struct FxCtx {
   int64_t v[3], h[3], P;        // own values at the common scales
   int Ev, Eh, EP;               // shifts of a neighbour's mantissas: E - e (biased)
   int L;                        // left shift of v_ij to the scale of u
-  uint32_t wrap_code;
-  int64_t wrap;
-  uint64_t near2, width, width_vv;  // r^2 - near2 < width: fixed point (0: never)
-  bool bottom;
+  PairRange R;                  // (width 0: fixed point never)
+  uint64_t width_vv;            // the same above kNearVV, for two viscous particles
 };
 
-// Entries t0, t0 + kLanes, ... of particle i below t1.
-template <int kPath>
-__device__ __forceinline__ void fx_loop(const FxCtx& C, const InstDev& P, const Fp64Buf& b,
-                                        const NbrWs& nw, int64_t n, int64_t i, uint32_t t0,
-                                        uint32_t t1, uint32_t* err, fx::Acc96 (&acc)[12],
-                                        double* slow, bool& any_slow) {
-  // the pressure's and the interfacial sums fit 64 bits (kMaxFx terms)
-  int64_t sp[3] = {0, 0, 0}, sx[3] = {0, 0, 0};
+// The entries that fixed point does not resolve, in FP64, after the common
+// loops have passed over them, by one lane in the list's order (so that the
+// sums do not depend on the number of lanes): viscous i, the pairs from vv on
+// are of two viscous particles.
+__device__ __noinline__ void slow_walk(int64_t n, int64_t i, uint32_t cnt, uint32_t vv,
+                                       const Fp64Buf* b, const InstDev* P, const NbrWs* nw,
+                                       const FxCtx* C, double* out) {
+  for (uint32_t t = 0; t < cnt; ++t) {
+    const uint32_t ent = nw->list[nbr_slot(n, i, t)], j = ent & kNbrIndexMask;
+    const PairVec v = pair_vec(C->q, nw->posq[j], ent, C->R);
+    const uint64_t r2 = fx::norm2(v.d[0], v.d[1], v.d[2]);
+    if (t >= vv ? r2 - kNearVV < C->width_vv : r2 - C->R.near2 < C->R.width) continue;
+    slow_pair(b, P, (uint32_t)i, j, v.across ? (C->R.bottom ? 1 : -1) : 0, out);
+  }
+}
+
+// Entries t0, t0 + kL, ... of particle i below t1.
+template <int kPath, int kL>
+__device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t n, int64_t i,
+                                        uint32_t t0, uint32_t t1, uint32_t* err,
+                                        fx::Acc96 (&acc)[12], bool& any_slow) {
   using fx::Half;
   using fx::mul;
   using fx::split;
+  // the pressure's and the interfacial sums fit 64 bits (kMaxFx terms)
+  int64_t sp[3] = {0, 0, 0}, sx[3] = {0, 0, 0};
   // the next entry's position record is loaded one entry ahead, the entry
   // after it two ahead
   if (t0 >= t1) return;
   uint32_t ent_n = nw.list[nbr_slot(n, i, t0)];
   QPos q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
-  uint32_t ent_nn = t0 + kLanes < t1 ? nw.list[nbr_slot(n, i, t0 + kLanes)] : ent_n;
-  for (uint32_t t = t0; t < t1; t += kLanes) {
+  uint32_t ent_nn = t0 + kL < t1 ? nw.list[nbr_slot(n, i, t0 + kL)] : ent_n;
+  for (uint32_t t = t0; t < t1; t += kL) {
     const uint32_t ent = ent_n;
     const uint32_t j = checked_index(ent & kNbrIndexMask, n, err);
     const QPos q = q_n;
     ent_n = ent_nn;
     q_n = ld_qpos(nw.posq + checked_index(ent_n & kNbrIndexMask, n, err));
-    if (t + 2 * kLanes < t1) ent_nn = nw.list[nbr_slot(n, i, t + 2 * kLanes)];
+    if (t + 2 * kL < t1) ent_nn = nw.list[nbr_slot(n, i, t + 2 * kL)];
     const PairRec* __restrict__ rec = nw.prec + j;
-    const bool across = (ent >> (kNbrIndexBits + 4)) == C.wrap_code;
-    int64_t dz = sub64(C.q.z, q.z);
-    if (across) dz = (int64_t)((uint64_t)dz + (uint64_t)C.wrap);
-    const Half d[3] = {split(sub64(C.q.x, q.x)), split(sub64(C.q.y, q.y)), split(dz)};
+    const PairVec pv = pair_vec(C.q, q, ent, C.R);
+    const Half(&d)[3] = pv.d;
     const uint64_t r2 = fx::norm2(d[0], d[1], d[2]);
-    const uint64_t near2 = kPath == kPathVV ? kNearVV : C.near2;
-    const uint64_t width = kPath == kPathVV ? C.width_vv : C.width;
-    if (r2 - near2 >= width) {
-      slow_pair(&b, &P, (uint32_t)i, j, across ? (C.bottom ? 1 : -1) : 0, slow);
+    if (kPath == kPathVV ? r2 - kNearVV >= C.width_vv : r2 - C.R.near2 >= C.R.width) {
       any_slow = true;
       continue;
     }
@@ -918,13 +1078,12 @@ __device__ __forceinline__ void add_lane(fx::Acc96& a, const fx::Acc96& give, in
   a.add3(x, y, z);
 }
 
-// The kLanes lanes' twelve sums added, lane l left with sums kKeep l ..
-// kKeep (l + 1) - 1 in acc[0 .. kKeep - 1]: each exchange halves what a lane
-// holds.
-constexpr int kKeep = 12 / kLanes;
+// The kL lanes' twelve sums added, lane l left with sums m l .. m (l + 1) - 1,
+// m = 12 / kL, in acc[0 .. m - 1]: each exchange halves what a lane holds.
+template <int kL>
 __device__ __forceinline__ void reduce12(fx::Acc96 (&acc)[12]) {
 #pragma unroll
-  for (int o = kLanes / 2, m = 6; o > 0; o >>= 1, m >>= 1) {
+  for (int o = kL / 2, m = 6; o > 0; o >>= 1, m >>= 1) {
     const bool up = (threadIdx.x & o) != 0;
 #pragma unroll
     for (int k = 0; k < m; ++k) {
@@ -935,16 +1094,16 @@ __device__ __forceinline__ void reduce12(fx::Acc96 (&acc)[12]) {
   }
 }
 
-template <int BLOCK>
+template <int BLOCK, int kL>
 __global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
 k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
             NbrWs nw, uint32_t* err, int64_t part_totals) {
-  constexpr int kRows = BLOCK / kLanes;
+  constexpr int kRows = BLOCK / kL, kKeep = 12 / kL;
   __shared__ double sums[kRows][kSlots + 1];
   const int64_t n_fluid = nw.part[part_totals + 1], n_inv = nw.part[part_totals];
   const int64_t first = (int64_t)blockIdx.x * kRows;
   if (first >= n_fluid) return;
-  const int row = threadIdx.x / kLanes, lane = threadIdx.x % kLanes;
+  const int row = threadIdx.x / kL, lane = threadIdx.x % kL;
   const bool live = first + row < n_fluid;
   const bool inv_i = first + row < n_inv;
   const int64_t i = live ? checked_index(nw.order[first + row], n, err) : 0;
@@ -954,29 +1113,44 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   C.q = ld_qpos(nw.posq + i);
   if (live) {
     cnt = checked_count(nw.count[i], nw.cap, err);
-    const uint32_t parts = nw.count_a[i];
-    na = min(parts & 0xFFFFu, cnt);
-    nb = min(parts >> 16, cnt - na);
+    const uint32_t parts = nw.parts[i];
+    na = min(part_inv(parts), cnt);
+    nb = min(part_vis(parts), cnt - na);
   }
   // first walk: the largest exponents, and the largest |v_ij|
   const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
   uint32_t eP = C.q.exps >> 16, ev = C.q.tag >> 16, eh = C.q.exps & 0xFFFFu;
   float dv = 0.f;
   const float4 vi = nw.pvel[i];
-  for (uint32_t t = lane; t < cnt; t += kLanes) {
-    const uint32_t j = checked_index(nw.list[nbr_slot(n, i, t)] & kNbrIndexMask, n, err);
-    const uint2 m = *reinterpret_cast<const uint2*>(&nw.posq[j].tag);
-    eP = max(eP, m.y >> 16);
-    if (t >= u0) {
-      ev = max(ev, m.x >> 16);
-      eh = max(eh, m.y & 0xFFFFu);
-      const float4 vj = nw.pvel[j];
-      const float x = fabsf(vi.x - vj.x), y = fabsf(vi.y - vj.y), z = fabsf(vi.z - vj.z);
-      dv = fmaxf(dv, fmaxf(x, fmaxf(y, z)));
+  for (uint32_t t0 = lane; t0 < cnt; t0 += 4 * kL) {  // four entries' loads in flight
+    uint32_t j[4];
+    uint2 m[4];
+    float4 vj[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      const uint32_t t = t0 + u * kL;
+      j[u] = t < cnt ? checked_index(nw.list[nbr_slot(n, i, t)] & kNbrIndexMask, n, err)
+                     : (uint32_t)i;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      m[u] = *reinterpret_cast<const uint2*>(&nw.posq[j[u]].tag);
+      if (t0 + u * kL >= u0) vj[u] = nw.pvel[j[u]];
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      eP = max(eP, m[u].y >> 16);
+      if (t0 + u * kL >= u0) {
+        ev = max(ev, m[u].x >> 16);
+        eh = max(eh, m[u].y & 0xFFFFu);
+        const float x = fabsf(vi.x - vj[u].x), y = fabsf(vi.y - vj[u].y),
+                    z = fabsf(vi.z - vj[u].z);
+        dv = fmaxf(dv, fmaxf(x, fmaxf(y, z)));
+      }
     }
   }
 #pragma unroll
-  for (int o = 1; o < kLanes; o <<= 1) {
+  for (int o = 1; o < kL; o <<= 1) {
     eP = max(eP, __shfl_xor_sync(~0u, eP, o));
     ev = max(ev, __shfl_xor_sync(~0u, ev, o));
     eh = max(eh, __shfl_xor_sync(~0u, eh, o));
@@ -995,14 +1169,9 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const bool covered = cnt <= kMaxFx && eP < 2047u && ev < 2047u && eh < 2047u &&
                        bound < 1e30f && (still || bound > 1e-30f);
   {
-    const int64_t g = (int64_t)cw.skey[i] / P.slabs;  // grid cell
-    const int cz_i = (int)((g - P.cell_base / P.slabs) / ((int64_t)P.nx * P.ny));
-    C.bottom = cz_i == 0;
-    C.wrap_code = !P.periodic_z ? 3u : (C.bottom ? 2u : (cz_i == P.nz - 1 ? 0u : 3u));
-    C.wrap = C.bottom ? P.fx_Hz : -P.fx_Hz;
-    C.near2 = P.fx_near;
-    C.width = covered ? P.fx_width : 0u;
-    C.width_vv = C.width ? C.width - (kNearVV - P.fx_near) : 0u;
+    C.R = pair_range(P, z_cell(P, cw.skey[i]));
+    if (!covered) C.R.width = 0u;
+    C.width_vv = C.R.width ? C.R.width - (kNearVV - C.R.near2) : 0u;
     const PairRec r = nw.prec[i];
     C.Ev = E_v1 + 1022;
     C.Eh = E2 - 2 + 1022;
@@ -1015,10 +1184,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     }
     C.P = shr(r.P, C.EP - (int)(C.q.exps >> 16));
   }
-  double slow[12];
   bool any_slow = false;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) slow[k] = 0.0;
   // the inviscid neighbours, the viscous ones, the walls
   const uint32_t end[4] = {0u, na, na + nb, cnt};
   const int phases = __syncthreads_or(live && cnt > na + nb) ? 3 : 2;
@@ -1026,35 +1192,40 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     fx::Acc96 acc[12];
     const uint32_t t0 = ph == 0 ? end[0] : (ph == 1 ? end[1] : end[2]);
     const uint32_t t1 = ph == 0 ? end[1] : (ph == 1 ? end[2] : end[3]);
+    if (!__any_sync(~0u, t0 < t1)) {  // none for this warp's particles
+#pragma unroll
+      for (int k = 0; k < kKeep; ++k) sums[row][12 * ph + kKeep * lane + k] = 0.0;
+      continue;
+    }
     if (inv_i) {
       if (ph == 0)
-        fx_loop<kPathII>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+        fx_loop<kPathII, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
       else
-        fx_loop<kPathIX>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
     } else {
       if (ph == 0)
-        fx_loop<kPathIX>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
       else
-        fx_loop<kPathVV>(C, P, b, nw, n, i, t0 + lane, t1, err, acc, slow, any_slow);
+        fx_loop<kPathVV, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
     }
     __syncwarp();
     if (ph == 0 && __all_sync(~0u, inv_i)) {  // pairs of inviscid particles: pressure alone
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
 #pragma unroll
-        for (int o = 1; o < kLanes; o <<= 1) add_lane(acc[k], acc[k], o);
+        for (int o = 1; o < kL; o <<= 1) add_lane(acc[k], acc[k], o);
       }
 #pragma unroll
-      for (int k = 0; k < 3; k += kLanes) {  // sum k + lane
+      for (int k = 0; k < 3; k += kL) {  // sum k + lane
         fx::Acc96 mine = acc[k];
 #pragma unroll
-        for (int q = 1; q < kLanes && k + q < 3; ++q)
+        for (int q = 1; q < kL && k + q < 3; ++q)
           if (lane == q) mine = acc[k + q];
         if (k + lane < 3) sums[row][k + lane] = mine.value(E_P - 57);
       }
       continue;
     }
-    reduce12(acc);
+    reduce12<kL>(acc);
     // the pressure's sums are in units of 2^(E_P - 57), the interfacial
     // force's of 2^-58, the torque's of 2^(E2 - 84), the others' of 2^(E2 - 83)
     const bool unlike = inv_i ? ph > 0 : ph == 0;
@@ -1068,11 +1239,14 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
 #pragma unroll
   for (int k = 0; k < kKeep; ++k) sums[row][36 + kKeep * lane + k] = 0.0;
   __syncwarp();
-  if (__any_sync(~0u, any_slow)) {  // the FP64 route's sums, lane by lane
-    for (int l = 0; l < kLanes; ++l) {
-      if (lane == l && any_slow)
-        for (int k = 0; k < 12; ++k) sums[row][36 + k] += slow[k];
-      __syncwarp();
+  if (__any_sync(~0u, any_slow)) {  // the FP64 route
+#pragma unroll
+    for (int o = 1; o < kL; o <<= 1) any_slow |= __shfl_xor_sync(~0u, (int)any_slow, o) != 0;
+    if (lane == 0 && any_slow) {
+      double slow[12];
+      for (int k = 0; k < 12; ++k) slow[k] = 0.0;
+      slow_walk(n, i, cnt, inv_i ? cnt : na, &b, &P, &nw, &C, slow);
+      for (int k = 0; k < 12; ++k) sums[row][36 + k] = slow[k];
     }
   }
   __syncthreads();
@@ -1208,23 +1382,20 @@ cudaError_t launch_density_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f
                                 const InstDev* inst, const CellWs& cw, const NbrWs& nw,
                                 uint32_t* err, cudaStream_t s, const LaunchCfg& lc,
                                 int* launches) {
-  const unsigned g32 = (unsigned)((n + 31) / 32), g64 = (unsigned)((n + 63) / 64),
-                 g128 = (unsigned)((n + 127) / 128);
-  if (lc.any_filter) {
+  const auto blocks = [&](int t) { return (unsigned)((n * kLanes + t - 1) / t); };
+  auto go = [&](auto filter) {
+    constexpr bool F = decltype(filter)::value;
     if (lc.block_density == 32)
-      k_density_fp64<32, true><<<g32, 32, 0, s>>>(n, b, f, inst, cw, nw, err);
+      k_density_fp64<32, F><<<blocks(32), 32, 0, s>>>(n, b, f, inst, cw, nw, err);
     else if (lc.block_density == 64)
-      k_density_fp64<64, true><<<g64, 64, 0, s>>>(n, b, f, inst, cw, nw, err);
+      k_density_fp64<64, F><<<blocks(64), 64, 0, s>>>(n, b, f, inst, cw, nw, err);
     else
-      k_density_fp64<128, true><<<g128, 128, 0, s>>>(n, b, f, inst, cw, nw, err);
-  } else {
-    if (lc.block_density == 32)
-      k_density_fp64<32, false><<<g32, 32, 0, s>>>(n, b, f, inst, cw, nw, err);
-    else if (lc.block_density == 64)
-      k_density_fp64<64, false><<<g64, 64, 0, s>>>(n, b, f, inst, cw, nw, err);
-    else
-      k_density_fp64<128, false><<<g128, 128, 0, s>>>(n, b, f, inst, cw, nw, err);
-  }
+      k_density_fp64<128, F><<<blocks(128), 128, 0, s>>>(n, b, f, inst, cw, nw, err);
+  };
+  if (lc.any_filter)
+    go(std::true_type());
+  else
+    go(std::false_type());
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -1243,13 +1414,20 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
   const int opt = (lc.any_literal ? kOptLiteral : 0) | (lc.any_collision ? kOptCollision : 0);
   if (opt == 0) {  // the default form, in fixed point
     k_pair_records<<<grid_for(n, 256, lc.sm_count, 32), 256, 0, s>>>(n, b, inst, nw);
-    const auto rows = [&](int block) { return (unsigned)((n * kLanes + block - 1) / block); };
-    if (lc.block_forces == 256)
-      k_forces_fx<256><<<rows(256), 256, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
-    else if (lc.block_forces == 64)
-      k_forces_fx<64><<<rows(64), 64, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    auto fixed = [&](auto lanes) {
+      constexpr int L = decltype(lanes)::value;
+      const auto blocks = [&](int t) { return (unsigned)((n * L + t - 1) / t); };
+      if (lc.block_forces == 256)
+        k_forces_fx<256, L><<<blocks(256), 256, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+      else if (lc.block_forces == 64)
+        k_forces_fx<64, L><<<blocks(64), 64, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+      else
+        k_forces_fx<128, L><<<blocks(128), 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    };
+    if (n < kPairLanes4)
+      fixed(std::integral_constant<int, 4>());
     else
-      k_forces_fx<128><<<rows(128), 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+      fixed(std::integral_constant<int, 2>());
     if (launches) *launches += 2;
     return cudaGetLastError();
   }

@@ -388,10 +388,8 @@ void carve(void* state, void* ws, int32_t n_inst, int64_t n, int64_t n_cells,
   c.nw.posq = precision == SPH_FP64 ? w.take<QPos>(n) : nullptr;
   c.nw.prec = precision == SPH_FP64 ? w.take<PairRec>(n) : nullptr;
   c.nw.pvel = precision == SPH_FP64 ? w.take<float4>(n) : nullptr;
-  c.nw.cls = precision == SPH_FP64 ? w.take<uint32_t>(n_cells / kSlabs * 2 * kMaxCandWords)
-                                   : nullptr;
   c.nw.mask = w.take<uint32_t>((int64_t)kMaxCandWords * n);
-  c.nw.ncand = w.take<uint32_t>(n_cells / kSlabs);
+  c.nw.ncand = w.take<uint32_t>(n_cells / kSlabs * (precision == SPH_FP64 ? 2 : 1));
   c.nw.cand = w.take<uint32_t>(n_cells / kSlabs * kMaxCand);
   c.nw.cap = cap;
   if (precision == SPH_MIXED) {  // the reused candidate lists of the mixed form
@@ -402,7 +400,7 @@ void carve(void* state, void* ws, int32_t n_inst, int64_t n, int64_t n_cells,
   if (precision == SPH_FP64) {
     c.f.vp = w.take<dvec2>(n);
     // the split lists and the species order of the FP64 pair pass
-    c.nw.count_a = w.take<uint32_t>(n);
+    c.nw.parts = w.take<uint32_t>(n);
     c.nw.order = w.take<uint32_t>(n);
     c.nw.part = w.take<uint32_t>(2 * ((n + kPartTile - 1) / kPartTile) + 2);
   } else {
@@ -544,10 +542,12 @@ sph_status enqueue_cells(sph_ctx* c, cudaStream_t s, int mode, int* launches,
 // the instances that rebuild in this step; null: all).
 sph_status enqueue_search(sph_ctx* c, cudaStream_t s, int* launches,
                           const InstState* gate = nullptr) {
-  const float4* rec = mixed(c) ? c->mf.oref : c->nw.posf;
-  const uint32_t* inst_of = mixed(c) ? c->mbuf[c->cur].inst : c->buf[c->cur].inst;
-  CK(launch_cell_search(mixed(c), c->n, rec, inst_of, c->inst, c->n_inst, c->max_cells, c->cw,
-                        c->nw, c->err, s, c->lc, launches, gate));
+  if (mixed(c))
+    CK(launch_cell_search(c->n, c->mf.oref, c->mbuf[c->cur].inst, c->inst, c->n_inst,
+                          c->max_cells, c->cw, c->nw, c->err, s, c->lc, launches, gate));
+  else
+    CK(launch_cell_search64(c->n, c->buf[c->cur], c->inst, c->n_inst, c->max_cells, c->cw, c->nw,
+                            c->err, s, c->lc, launches));
   return SPH_OK;
 }
 
@@ -1218,13 +1218,19 @@ sph_status sph_get_neighbors(sph_ctx* c, int64_t* offsets, int64_t* nbr, int64_t
                      sizeof(uint32_t) * n, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaMemcpyAsync(list.data(), c->nw.list, sizeof(uint32_t) * list.size(),
                      cudaMemcpyDeviceToHost, c->stream));
+  std::vector<uint32_t> parts;  // FP64 form: with the entries beyond 2h
+  if (!mixed(c)) {
+    parts.resize((size_t)n);
+    CK(cudaMemcpyAsync(parts.data(), c->nw.parts, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost,
+                       c->stream));
+  }
   sph_status st = sph_check(c);
   std::vector<int64_t> where((size_t)n);
   for (int64_t k = 0; k < n; ++k) where[id[k]] = k;
   int64_t tot = 0;
   for (int64_t o = 0; o < n; ++o) {
     offsets[o] = tot;
-    tot += cnt[(size_t)where[o]];
+    tot += cnt[(size_t)where[o]] - (parts.empty() ? 0u : part_dead(parts[(size_t)where[o]]));
   }
   offsets[n] = tot;
   if (!nbr || cap < tot) return st != SPH_OK ? st : SPH_ERR_ARG;
@@ -1232,8 +1238,10 @@ sph_status sph_get_neighbors(sph_ctx* c, int64_t* offsets, int64_t* nbr, int64_t
   for (int64_t o = 0; o < n; ++o) {
     const int64_t k = where[o];
     tmp.clear();
-    for (uint32_t t = 0; t < cnt[(size_t)k]; ++t)
-      tmp.push_back(id[list[(size_t)nbr_slot(n, k, t)] & kNbrIndexMask]);
+    for (uint32_t t = 0; t < cnt[(size_t)k]; ++t) {
+      const uint32_t j = list[(size_t)nbr_slot(n, k, t)] & kNbrIndexMask;
+      if ((int64_t)j != k) tmp.push_back(id[j]);  // (the FP64 form's entries beyond 2h name k)
+    }
     std::sort(tmp.begin(), tmp.end());
     for (size_t t = 0; t < tmp.size(); ++t) nbr[offsets[o] + (int64_t)t] = tmp[t];
   }

@@ -22,7 +22,7 @@ constexpr int kReduceChunk = 32768;    // particles per partial of the plain-arr
 constexpr int kStateChunk = 8192;      // particles per partial of the state's FP64 reductions
 constexpr int kDiagFields = 24;        // doubles per diagnostics partial
 constexpr int kMaxInst = 65535;
-constexpr int kSlabs = 4;              // x-slabs per cell in the sort key
+constexpr int kSlabs = 4;              // parts per cell in the sort key
 
 // Error bits latched on the device.
 enum : uint32_t {
@@ -65,7 +65,8 @@ struct InstDev {
   int32_t alphaP;                 // integer Tait exponent
   uint32_t flags;
   int32_t periodic_z;
-  int32_t slabs;                  // x-slabs per cell: sort key = cell * slabs + slab
+  int32_t slabs;                  // parts per cell: sort key = cell * slabs + part, the
+                                  // x-slab (mixed form) or the species class (FP64 form)
   int64_t cell_base;              // first global sort key of the instance
   int64_t p_begin, p_end;         // particle range (fixed across sorts)
   int64_t chunk_base;             // first reduction chunk of the instance
@@ -201,9 +202,12 @@ struct CellWs {
 // cell displacement code (dx+1) | (dy+1) << 2 | (dz+1) << 4 of the particle's
 // cell relative to the candidate's (used by the mixed form).  Per particle it
 // writes one bit per candidate of its cell: word k of particle i, at
-// mask[k * n + i], covers candidates 32k .. 32k + 31.  The density pass walks
-// the set bits in order (the FP64 form re-tests each exactly) and writes the
-// neighbours as i's neighbour list for the pair pass.
+// mask[k * n + i], covers candidates 32k .. 32k + 31, from which the reused
+// lists (mixed form) and the density pass's lists (FP64 form) are built.
+// the fields of NbrWs::parts
+__host__ __device__ __forceinline__ uint32_t part_inv(uint32_t p) { return p & 0x7FFu; }
+__host__ __device__ __forceinline__ uint32_t part_vis(uint32_t p) { return (p >> 11) & 0x7FFu; }
+__host__ __device__ __forceinline__ uint32_t part_dead(uint32_t p) { return p >> 22; }
 constexpr uint32_t kNbrIndexBits = 26;
 constexpr uint32_t kNbrIndexMask = (1u << kNbrIndexBits) - 1u;
 constexpr int64_t kMaxParticles = (int64_t)1 << kNbrIndexBits;  // 67,108,864
@@ -216,7 +220,6 @@ constexpr int kMaxCandWords = kMaxCand / 32;
 // writes whole sectors and reads 1 KB contiguous per group.  An entry is a
 // candidate-table entry (index | displacement code).
 constexpr int kNbrGroup = 8;
-constexpr uint32_t kHasWall = 0x80000000u;
 constexpr int kPartTile = 4096;  // particles per tile of the species partition
 
 // Compile-time options of the pair pass (template argument kOpt).
@@ -231,24 +234,22 @@ struct NbrWs {
   uint32_t* list;       // neighbour entries, layout above
   uint32_t* count;      // neighbours per particle (list length)
   // FP64 form: a particle's list holds its inviscid neighbours, then the
-  // viscous ones, then the walls; count_a packs the numbers of the first two
-  // (low and high 16 bits).  Species partition of the fluid particles for
+  // viscous ones, then the walls, as the search's prefilter finds them; an
+  // entry that the density pass finds beyond 2h names the particle itself.  parts packs the entries of the first two classes (11 bits each)
+  // and the entries beyond 2h (10 bits).  Species partition of the fluid particles for
   // the pair pass: order[0 .. n_inv) inviscid, then the viscous ones, each in
   // sorted order.
-  uint32_t* count_a;
+  uint32_t* parts;
   uint32_t* order;
   uint32_t* part;       // per-tile counts of the partition, then its totals
   float4* posf;         // FP32 copy of sorted positions (FP64-form prefilter)
   QPos* posq;           // fixed-point copy of sorted positions (FP64 form)
   PairRec* prec;        // fixed-point pair records (FP64 form)
   float4* pvel;         // FP32 velocities, for the pair pass's scales (FP64 form)
-  // FP64 form: per grid cell the inviscid candidates of its table (32 words of
-  // bits in table order), then the wall candidates (32 words).
-  uint32_t* cls;
   uint32_t* mask;       // [kMaxCandWords][n] candidate hit bits
   uint32_t* cand;       // [grid cells][kMaxCand] candidate table of each cell
-  uint32_t* ncand;      // [grid cells] candidates of each cell (FP64 form: kHasWall
-                        // set if some are walls)
+  uint32_t* ncand;      // [grid cells] candidates of each cell (FP64 form: two words, the
+                        // second with the ends of the first two species classes)
   // Pressure filter only (null otherwise): the kernel shape t^4 (2q + 1) of
   // every list entry, written by the density pass in the list's layout
   // (nbr_slot), so the filter neither gathers positions nor re-evaluates W.
@@ -349,59 +350,6 @@ struct MaskWalk {
 #pragma unroll
     for (int u = 0; u < B; ++u) {
       while (w == 0u && k + 1 < K) w = sw[++k * stride];
-      if (w != 0u) {
-        const uint32_t bit = (uint32_t)__ffs(w) - 1u;
-        w &= w - 1u;
-        e[u] = tab[(k << 5) + bit];
-        m = (uint32_t)u + 1u;
-      }
-    }
-    return m;
-  }
-};
-
-// The same walk over one species class at a time, in the FP64 form: class 0
-// the inviscid candidates, 1 the viscous ones, 2 the walls, told apart by the
-// cell's class words, so that a list comes out sorted by class with one
-// writer and no entry is set aside.
-struct ClassWalk {
-  const uint32_t* __restrict__ tab;
-  const uint32_t* __restrict__ cls;
-  uint32_t* sw;
-  uint32_t stride, K, k = 0, w = 0;
-  int c = 0;
-  bool walls;
-  __device__ __forceinline__ ClassWalk(const NbrWs& nw, int64_t n, int64_t i, int64_t g,
-                                       uint32_t* sw_, uint32_t stride_)
-      : tab(nw.cand + g * kMaxCand), cls(nw.cls + g * 2 * kMaxCandWords), sw(sw_),
-        stride(stride_) {
-    const uint32_t nc = nw.ncand[g];
-    walls = (nc & kHasWall) != 0u;
-    K = ((nc & ~kHasWall) + 31u) >> 5;
-    const uint32_t* __restrict__ mw = nw.mask + i;
-#pragma unroll 4
-    for (uint32_t t = 0; t < K; ++t) sw[t * stride] = mw[(int64_t)t * n];
-  }
-  __device__ __forceinline__ uint32_t word() const {
-    const uint32_t m = sw[k * stride];
-    if (c == 0) return m & cls[k];
-    if (c == 2) return m & cls[kMaxCandWords + k];
-    return m & ~(cls[k] | cls[kMaxCandWords + k]);
-  }
-  __device__ __forceinline__ void start(int c_) {
-    c = c_;
-    k = 0;
-    w = K ? word() : 0u;
-  }
-  template <int B>
-  __device__ __forceinline__ uint32_t next(uint32_t (&e)[B]) {
-    uint32_t m = 0;
-#pragma unroll
-    for (int u = 0; u < B; ++u) {
-      while (w == 0u && k + 1 < K) {
-        ++k;
-        w = word();
-      }
       if (w != 0u) {
         const uint32_t bit = (uint32_t)__ffs(w) - 1u;
         w &= w - 1u;

@@ -32,20 +32,24 @@ cudaError_t launch_scatter_sort(const CellWs& cw, const uint32_t* id, int64_t n,
                                 const uint32_t* gate = nullptr);
 
 // ---- neighbour search (sph_search.cu) ---------------------------------------
-// One warp per cell of every instance (grid.y = instance); writes the
-// candidate tables and candidate masks of nw, from which the density pass
-// builds the neighbour lists.  rec: the per-particle FP32 records (mixed: cell offset
-// and species, FP64 form: the rounded position and species).  mixed_form:
-// exact FP32 test with cell-displacement codes; otherwise the FP32 prefilter.
+// Mixed form.  One warp per cell of every instance (grid.y = instance); writes
+// the candidate tables and candidate masks of nw, from which the reused lists
+// are built.  rec: the per-particle FP32 records (cell offset and species); an
+// exact FP32 test r^2 < (2h + skin)^2 with cell-displacement codes.
 // lc.search_warps = 0 selects the thread-per-particle mapping (inst_of: the
 // instance of each sorted particle), which writes the same output.
-// gate (mixed form): only the instances whose InstState::rebuild is set are
-// searched (null: all).  The mixed form's test is r^2 < (2h + skin)^2.
-cudaError_t launch_cell_search(bool mixed_form, int64_t n, const float4* rec,
-                               const uint32_t* inst_of, const InstDev* inst, int32_t n_inst,
-                               int64_t max_cells, const CellWs& cw, const NbrWs& nw,
-                               uint32_t* err, cudaStream_t s, const LaunchCfg& lc,
-                               int* launches, const InstState* gate = nullptr);
+// gate: only the instances whose InstState::rebuild is set are searched
+// (null: all).
+cudaError_t launch_cell_search(int64_t n, const float4* rec, const uint32_t* inst_of,
+                               const InstDev* inst, int32_t n_inst, int64_t max_cells,
+                               const CellWs& cw, const NbrWs& nw, uint32_t* err, cudaStream_t s,
+                               const LaunchCfg& lc, int* launches, const InstState* gate);
+// FP64 form: the same two mappings with the FP32 prefilter on the rounded
+// positions, the candidates in class order.
+cudaError_t launch_cell_search64(int64_t n, const Fp64Buf& b, const InstDev* inst,
+                                 int32_t n_inst, int64_t max_cells, const CellWs& cw,
+                                 const NbrWs& nw, uint32_t* err, cudaStream_t s,
+                                 const LaunchCfg& lc, int* launches);
 // Raise the dynamic shared-memory limit of the search kernels (once, before
 // any launch or stream capture).
 cudaError_t prepare_search_kernels();

@@ -48,6 +48,10 @@ struct Fp64View {
     return b.vel[i].w * inv_m;
   }
   __device__ __forceinline__ double pres(int64_t i) const { return f.P[i]; }
+  // Neighbours of particle i (its list's entries but those beyond 2h).
+  __device__ __forceinline__ uint32_t neighbours(const NbrWs& nw, int64_t i) const {
+    return nw.count[i] - part_dead(nw.parts[i]);
+  }
   // The wall torque record of particle i, whether it is not zero (it is zero
   // for every particle without a wall neighbour, walls included; the test
   // looks at the bits, so that no FP64 instruction is spent on the zeros),
@@ -101,6 +105,9 @@ struct MixView {
     return 1.0 / rho;
   }
   __device__ __forceinline__ double pres(int64_t i) const { return (double)f.P[i]; }
+  __device__ __forceinline__ uint32_t neighbours(const NbrWs& nw, int64_t i) const {
+    return nw.count[i];
+  }
   // The wall torque record of particle i (see Fp64View).
   typedef float4 TwRec;
   __device__ __forceinline__ TwRec tw(int64_t i) const { return f.tw[i]; }
@@ -296,7 +303,7 @@ k_diag_chunks(int32_t n_inst, const InstDev* __restrict__ inst, View V, NbrWs nw
     v[12] += 0.5 * m * u2;
     v[13] += 0.5 * I * (w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
     v[14] += m * tait_energy(P, rho, inv_rho, ecoef);
-    pairs += nw.count[i];
+    pairs += V.neighbours(nw, i);
     const long long rb = dbits(rho), ub = dbits(u2);
     rmin_b = rb < rmin_b ? rb : rmin_b;
     rmax_b = rb > rmax_b ? rb : rmax_b;
@@ -417,6 +424,7 @@ k_breakdown_chunks(int32_t n_inst, int64_t n, const InstDev* __restrict__ inst, 
     for (uint32_t t = 0; t < cnt; ++t) {
       uint32_t j = nw.list[nbr_slot(n, i, t)] & kNbrIndexMask;
       if ((int64_t)j >= n) j = 0;
+      if ((int64_t)j == i) continue;  // (FP64 form: an entry beyond 2h)
       double pj[3], vj[3], wj[3];
       V.pos(j, P, pj);
       V.vel(j, vj);
@@ -518,6 +526,7 @@ k_census_chunks(int32_t n_inst, int64_t n, const InstDev* __restrict__ inst, Vie
     for (uint32_t t = 0; t < cnt; ++t) {
       uint32_t j = nw.list[nbr_slot(n, i, t)] & kNbrIndexMask;
       if ((int64_t)j >= n) j = 0;
+      if ((int64_t)j == i) continue;  // (FP64 form: an entry beyond 2h)
       const int sp_j = V.species(j);
       const int k = sp_j >= 2 ? (sp_i == 0 ? 3 : 4) : (sp_i + sp_j == 0 ? 0 : (sp_i + sp_j == 1 ? 1 : 2));
       c[k] += 1u;
