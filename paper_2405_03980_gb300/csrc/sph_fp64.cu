@@ -167,7 +167,7 @@ __global__ void k_reorder_fp64(int64_t n, Fp64Buf src, Fp64Buf dst, CellWs cw, N
                                const InstDev* __restrict__ inst) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t j = checked_index(cw.perm[k], n, cw.err);
+    const uint32_t j = checked_index(cw.slot[k], n, cw.err);
     const dvec4 p = src.pos[j];
     dst.pos[k] = p;
     dst.vel[k] = src.vel[j];
@@ -198,11 +198,11 @@ __device__ __forceinline__ bool inviscid(double w) { return __double2hiint(w) ==
 __device__ __forceinline__ bool is_wall(double w) { return __double2hiint(w) >= 0x40000000; }
 // Species classes and wall-row zeroing of the FP64 state, for the partition.
 struct Fp64Species {
-  Fp64Buf b;
+  const uint32_t* skey;
   Fp64Fields f;
   __device__ __forceinline__ int cls(int64_t i) const {  // 0 inviscid, 1 viscous, 2 wall
-    const double w = b.pos[i].w;
-    return inviscid(w) ? 0 : (is_wall(w) ? 2 : 1);
+    const int part = (int)(skey[i] & (uint32_t)(kSlabs - 1));  // (a cell's parts: cell_key)
+    return part < 2 ? 0 : part - 1;
   }
   __device__ __forceinline__ void zero(int64_t i) const {
     const dvec4 z = {0.0, 0.0, 0.0, 0.0};
@@ -834,7 +834,7 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // rounded at 2^-57 of the largest pressure.  A sum is exact: it does not
 // depend on the order of the list or on the number of lanes.
 //
-// kL lanes take a particle's entries in turn, two or four of them (warps of 16
+// kL lanes take a particle's entries in turn, two to eight of them (warps of 16
 // or 8 particles diverge less than warps of 32, and small vessels spread over
 // more warps; see kPairLanes4); their sums are added by shuffles and the block's first threads finish one
 // particle each, so the FP64 instructions of the end are issued by full
@@ -850,9 +850,11 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // (4.1e-16 to 8.1e-16), of the density 7e-17 (3.6e-16).  20.1M particles:
 // 134.3 ms before, 38.6 ms now.
 
-// Particles below which four lanes take a list, else two: four fill the GPU
-// sooner, two spend less on adding up (pair pass with 4 / 2 lanes: 8,960
-// particles 78 / 122 us, 2.5M 5.23 / 4.80 ms).
+// Particles below which eight and four lanes take a list, else two: more lanes
+// fill the GPU sooner, fewer spend less on adding up (pair pass with 8 / 4 / 2
+// lanes: 10,800 particles 58 / 73 / 124 us; with 4 / 2 169,000 369 / 376 us, 348,000 735 /
+// 718 us, 2.5M 5.23 / 4.80 ms).
+constexpr int64_t kPairLanes8 = 1 << 15;
 constexpr int64_t kPairLanes4 = 1 << 18;
 constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip
 // Entries that a 64-bit sum holds: a pressure term is below 2 (27/256) 2^57 (t^3 (1 - t) is at
@@ -1084,6 +1086,11 @@ template <int kL>
 __device__ __forceinline__ void reduce12(fx::Acc96 (&acc)[12]) {
 #pragma unroll
   for (int o = kL / 2, m = 6; o > 0; o >>= 1, m >>= 1) {
+    if (m == 1) {  // eight lanes: three sums are added up by both lanes of a pair
+#pragma unroll
+      for (int k = 0; k < 3; ++k) add_lane(acc[k], acc[k], o);
+      break;
+    }
     const bool up = (threadIdx.x & o) != 0;
 #pragma unroll
     for (int k = 0; k < m; ++k) {
@@ -1098,12 +1105,13 @@ template <int BLOCK, int kL>
 __global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
 k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
             NbrWs nw, uint32_t* err, int64_t part_totals) {
-  constexpr int kRows = BLOCK / kL, kKeep = 12 / kL;
+  constexpr int kRows = BLOCK / kL, kKeep = kL == 8 ? 3 : 12 / kL;
   __shared__ double sums[kRows][kSlots + 1];
   const int64_t n_fluid = nw.part[part_totals + 1], n_inv = nw.part[part_totals];
   const int64_t first = (int64_t)blockIdx.x * kRows;
   if (first >= n_fluid) return;
   const int row = threadIdx.x / kL, lane = threadIdx.x % kL;
+  const int part = kL == 8 ? lane >> 1 : lane;  // which of the sums the lane keeps
   const bool live = first + row < n_fluid;
   const bool inv_i = first + row < n_inv;
   const int64_t i = live ? checked_index(nw.order[first + row], n, err) : 0;
@@ -1194,7 +1202,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     const uint32_t t1 = ph == 0 ? end[1] : (ph == 1 ? end[2] : end[3]);
     if (!__any_sync(~0u, t0 < t1)) {  // none for this warp's particles
 #pragma unroll
-      for (int k = 0; k < kKeep; ++k) sums[row][12 * ph + kKeep * lane + k] = 0.0;
+      for (int k = 0; k < kKeep; ++k) sums[row][12 * ph + kKeep * part + k] = 0.0;
       continue;
     }
     if (inv_i) {
@@ -1231,13 +1239,13 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     const bool unlike = inv_i ? ph > 0 : ph == 0;
 #pragma unroll
     for (int k = 0; k < kKeep; ++k) {
-      const int q = kKeep * lane + k;
+      const int q = kKeep * part + k;
       const int e = q < 3 ? E_P - 57 : (q < 6 ? (unlike ? -58 : E2 - 83) : (q < 9 ? E2 - 83 : E2 - 84));
       sums[row][12 * ph + q] = acc[k].value(e);
     }
   }
 #pragma unroll
-  for (int k = 0; k < kKeep; ++k) sums[row][36 + kKeep * lane + k] = 0.0;
+  for (int k = 0; k < kKeep; ++k) sums[row][36 + kKeep * part + k] = 0.0;
   __syncwarp();
   if (__any_sync(~0u, any_slow)) {  // the FP64 route
 #pragma unroll
@@ -1405,8 +1413,8 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
                                uint32_t* err, cudaStream_t s, const LaunchCfg& lc,
                                int* launches) {
   // the species partition of the fluid particles, then the pair pass over it
-  const int64_t nt = (n + kPartTile - 1) / kPartTile;
-  cudaError_t e = launch_partition(n, Fp64Species{b, f}, nw, s, launches);
+  const int64_t nt = part_tiles(n);
+  cudaError_t e = launch_partition(n, Fp64Species{cw.skey, f}, nw, s, launches);
   if (e != cudaSuccess) return e;
   const unsigned g256 = (unsigned)((n + 255) / 256), g128 = (unsigned)((n + 127) / 128),
                  g64 = (unsigned)((n + 63) / 64);
@@ -1424,7 +1432,9 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
       else
         k_forces_fx<128, L><<<blocks(128), 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
     };
-    if (n < kPairLanes4)
+    if (n < kPairLanes8)
+      fixed(std::integral_constant<int, 8>());
+    else if (n < kPairLanes4)
       fixed(std::integral_constant<int, 4>());
     else
       fixed(std::integral_constant<int, 2>());

@@ -451,7 +451,8 @@ sph_status plan(int32_t n_inst, const sph_params* params, const int64_t* counts,
     d.p_begin = pb;
     d.p_end = pb + counts[k];
     d.chunk_base = kb;
-    d.n_chunks = (counts[k] + kStateChunk - 1) / kStateChunk;
+    d.chunk = counts[k] < kSmallState ? kSmallStateChunk : kStateChunk;
+    d.n_chunks = (counts[k] + d.chunk - 1) / d.chunk;
     cb += (int64_t)d.nx * d.ny * d.nz * d.slabs;
     pb += counts[k];
     kb += d.n_chunks;

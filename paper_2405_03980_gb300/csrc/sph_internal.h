@@ -19,7 +19,12 @@ struct alignas(16) dvec2 {
 
 constexpr int kScanChunk = 4096;       // elements per block of the cell-count scan
 constexpr int kReduceChunk = 32768;    // particles per partial of the plain-array diagnostics
-constexpr int kStateChunk = 8192;      // particles per partial of the state's FP64 reductions
+// Particles per partial of the state's FP64 reductions, by the instance's own
+// size (so that a batched instance's sums equal its solo run's): a small vessel
+// gets enough blocks (10,800 particles in two chunks of 8192 took 15 us for
+// the wall torque), a large one even waves.
+constexpr int kStateChunk = 8192, kSmallStateChunk = 1024;
+constexpr int64_t kSmallState = 1 << 18;
 constexpr int kDiagFields = 24;        // doubles per diagnostics partial
 constexpr int kMaxInst = 65535;
 constexpr int kSlabs = 4;              // parts per cell in the sort key
@@ -70,7 +75,7 @@ struct InstDev {
   int64_t cell_base;              // first global sort key of the instance
   int64_t p_begin, p_end;         // particle range (fixed across sorts)
   int64_t chunk_base;             // first reduction chunk of the instance
-  int64_t n_chunks;
+  int64_t n_chunks, chunk;        // number and size of its chunks
   // ---- FP32 copies for the mixed form ----
   float cellf[3];                 // cell side per axis
   float lof[3];                   // grid origin lo per axis
@@ -184,8 +189,9 @@ constexpr uint32_t kCellBitsX = 11, kCellBitsY = 11, kCellBitsZ = 10;
 
 struct CellWs {
   uint32_t* key;        // global cell of each particle (pre-sort order)
-  uint32_t* slot;       // arrival slot within the cell (atomic order)
-  uint32_t* perm;       // sorted position -> pre-sort index
+  uint32_t* slot;       // arrival slot within the cell (atomic order); after the
+                        // sort: sorted position -> pre-sort index
+  uint32_t* perm;       // the same with the cells in arrival order
   uint32_t* skey;       // key in sorted order
   uint32_t* count;      // particles per cell
   uint32_t* start;      // exclusive scan of count, n_cells + 1 entries
@@ -220,7 +226,7 @@ constexpr int kMaxCandWords = kMaxCand / 32;
 // writes whole sectors and reads 1 KB contiguous per group.  An entry is a
 // candidate-table entry (index | displacement code).
 constexpr int kNbrGroup = 8;
-constexpr int kPartTile = 4096;  // particles per tile of the species partition
+constexpr int kPartTile = 1024;  // smallest tile of the species partition
 
 // Compile-time options of the pair pass (template argument kOpt).
 constexpr int kOptLiteral = 1;    // literal F_sn on v_ij (SPH_SN_LITERAL)

@@ -26,7 +26,8 @@ struct LaunchCfg {
 // *gate is zero (null: always run).
 cudaError_t launch_scan(const CellWs& cw, cudaStream_t s, const LaunchCfg& lc, int* launches,
                         const uint32_t* gate = nullptr);
-// perm[start[key[i]] + slot[i]] = i, then sort each cell by particle id.
+// perm[start[key[i]] + slot[i]] = i, then each cell part sorted by particle id
+// into cw.slot.
 cudaError_t launch_scatter_sort(const CellWs& cw, const uint32_t* id, int64_t n,
                                 cudaStream_t s, const LaunchCfg& lc, int* launches,
                                 const uint32_t* gate = nullptr);

@@ -371,7 +371,7 @@ __global__ void k_reorder_mixed(int64_t n, MixBuf src, MixBuf dst, CellWs cw,
   if (gate_closed(gate)) return;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t j = checked_index(cw.perm[k], n, cw.err);
+    const uint32_t j = checked_index(cw.slot[k], n, cw.err);
     dst.cell[k] = src.cell[j];
     dst.off[k] = src.off[j];
     float4 v, w;

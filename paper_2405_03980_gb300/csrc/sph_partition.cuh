@@ -1,5 +1,5 @@
 // Stable, deterministic partition of the fluid particles by species for the
-// pair passes (no atomics): per tile of kPartTile sorted particles the
+// pair passes (no atomics): per tile of sorted particles the
 // counts of inviscid and viscous fluid; their exclusive scans over the tiles
 // (inviscid first); then each tile writes its particles' indices in order,
 // nw.order[0 .. n_inv) the inviscid ones and nw.order[n_inv .. n_fluid) the
@@ -14,7 +14,11 @@ namespace sphgb {
 namespace {
 
 constexpr int kPartThreads = 256;
-constexpr int kPartPer = kPartTile / kPartThreads;  // 16 consecutive particles per thread
+// Consecutive particles per thread: 16, or 4 for fewer than kPartSmall
+// particles, whose tiles would leave the GPU idle (three blocks at 10,800
+// particles: 20 us for the partition).
+constexpr int kPartPer = 16, kPartPerSmall = kPartTile / kPartThreads;
+constexpr int64_t kPartSmall = 1 << 20;
 
 // Exclusive block scan of two counts at once (kPartThreads threads).
 __device__ __forceinline__ void block_scan2(uint32_t a, uint32_t v, uint32_t& ea, uint32_t& ev,
@@ -64,12 +68,12 @@ __device__ __forceinline__ void block_scan2(uint32_t a, uint32_t v, uint32_t& ea
   __syncthreads();
 }
 
-template <class View>
+template <int kPer, class View>
 __global__ void __launch_bounds__(kPartThreads)
 k_part_count(int64_t n, View V, uint32_t* __restrict__ part) {
-  const int64_t base = (int64_t)blockIdx.x * kPartTile + (int64_t)threadIdx.x * kPartPer;
+  const int64_t base = ((int64_t)blockIdx.x * kPartThreads + threadIdx.x) * kPer;
   uint32_t a = 0, v = 0;
-  for (int k = 0; k < kPartPer; ++k)
+  for (int k = 0; k < kPer; ++k)
     if (base + k < n) {
       const int c = V.cls(base + k);
       a += c == 0;
@@ -116,15 +120,15 @@ k_part_scan(int64_t nt, uint32_t* __restrict__ part) {
   }
 }
 
-template <class View>
+template <int kPer, class View>
 __global__ void __launch_bounds__(kPartThreads)
 k_part_scatter(int64_t n, View V, const uint32_t* __restrict__ part,
                uint32_t* __restrict__ order) {
-  const int64_t base = (int64_t)blockIdx.x * kPartTile + (int64_t)threadIdx.x * kPartPer;
-  int cls[kPartPer];
+  const int64_t base = ((int64_t)blockIdx.x * kPartThreads + threadIdx.x) * kPer;
+  int cls[kPer];
   uint32_t a = 0, v = 0;
 #pragma unroll
-  for (int k = 0; k < kPartPer; ++k) {
+  for (int k = 0; k < kPer; ++k) {
     cls[k] = base + k < n ? V.cls(base + k) : 3;
     a += cls[k] == 0;
     v += cls[k] == 1;
@@ -133,7 +137,7 @@ k_part_scatter(int64_t n, View V, const uint32_t* __restrict__ part,
   block_scan2(a, v, ea, ev, ta, tv);
   uint32_t oa = part[2 * blockIdx.x] + ea, ov = part[2 * blockIdx.x + 1] + ev;
 #pragma unroll
-  for (int k = 0; k < kPartPer; ++k) {
+  for (int k = 0; k < kPer; ++k) {
     const int64_t i = base + k;
     if (cls[k] == 0) order[oa++] = (uint32_t)i;
     else if (cls[k] == 1) order[ov++] = (uint32_t)i;
@@ -141,13 +145,23 @@ k_part_scatter(int64_t n, View V, const uint32_t* __restrict__ part,
   }
 }
 
+inline int64_t part_tiles(int64_t n) {
+  const int64_t tile = kPartThreads * (n < kPartSmall ? kPartPerSmall : kPartPer);
+  return (n + tile - 1) / tile;
+}
+
 template <class View>
 cudaError_t launch_partition(int64_t n, const View& V, const NbrWs& nw, cudaStream_t s,
                              int* launches) {
-  const int64_t nt = (n + kPartTile - 1) / kPartTile;
-  k_part_count<View><<<(unsigned)nt, kPartThreads, 0, s>>>(n, V, nw.part);
+  const int64_t nt = part_tiles(n);
+  const unsigned g = (unsigned)nt;
+  if (n < kPartSmall) k_part_count<kPartPerSmall><<<g, kPartThreads, 0, s>>>(n, V, nw.part);
+  else k_part_count<kPartPer><<<g, kPartThreads, 0, s>>>(n, V, nw.part);
   k_part_scan<<<1, kPartThreads, 0, s>>>(nt, nw.part);
-  k_part_scatter<View><<<(unsigned)nt, kPartThreads, 0, s>>>(n, V, nw.part, nw.order);
+  if (n < kPartSmall)
+    k_part_scatter<kPartPerSmall><<<g, kPartThreads, 0, s>>>(n, V, nw.part, nw.order);
+  else
+    k_part_scatter<kPartPer><<<g, kPartThreads, 0, s>>>(n, V, nw.part, nw.order);
   if (launches) *launches += 3;
   return cudaGetLastError();
 }

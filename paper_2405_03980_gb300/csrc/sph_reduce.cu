@@ -3,8 +3,8 @@
 // diagnostics (total mass M = M_s + M_n of Sec. 2.1, momentum, orbital and spin
 // angular momentum, energies).  Both state forms are read in FP64.
 //
-// Each instance's particle range is cut into fixed chunks of kStateChunk
-// particles counted from the instance's first particle (small enough that
+// Each instance's particle range is cut into fixed chunks (kStateChunk or
+// kSmallStateChunk particles) counted from the instance's first particle (small enough that
 // the chunks of a 20M-particle state fill the GPU in several even waves);
 // one block reduces one chunk in a fixed tree order and a second kernel adds
 // the chunk partials of an instance in a fixed order.  The result therefore depends only on the
@@ -128,14 +128,17 @@ struct ChunkRange {
 
 __device__ __forceinline__ ChunkRange chunk_range(const InstDev* inst, int32_t n_inst,
                                                   int64_t c) {
-  // instances are few; a linear scan keeps this simple and exact
-  int32_t k = 0;
-  while (k + 1 < n_inst && inst[k + 1].chunk_base <= c) ++k;
+  int32_t k = 0, hi = n_inst - 1;  // the last instance whose first chunk is <= c
+  while (k < hi) {
+    const int32_t mid = (k + hi + 1) >> 1;
+    if (inst[mid].chunk_base <= c) k = mid;
+    else hi = mid - 1;
+  }
   const InstDev& P = inst[k];
   ChunkRange r;
   r.inst = k;
-  r.begin = P.p_begin + (c - P.chunk_base) * (int64_t)kStateChunk;
-  r.end = r.begin + kStateChunk;
+  r.begin = P.p_begin + (c - P.chunk_base) * P.chunk;
+  r.end = r.begin + P.chunk;
   if (r.end > P.p_end) r.end = P.p_end;
   return r;
 }
@@ -194,6 +197,12 @@ k_wall_torque_chunks(int32_t n_inst, const InstDev* __restrict__ inst, View V,
       v[2] += t[2];
     }
   }
+  // (a chunk away from the walls has nothing to add up)
+  const bool some = v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || isnan(v[0] + v[1] + v[2]);
+  if (!__syncthreads_or(some)) {
+    if (threadIdx.x < 3) partials[(int64_t)blockIdx.x * 3 + threadIdx.x] = 0.0;
+    return;
+  }
   block_sum<3>(v, sh);
   if (threadIdx.x < 3)
     partials[(int64_t)blockIdx.x * 3 + threadIdx.x] = sh[threadIdx.x * kRedThreads];
@@ -209,6 +218,7 @@ __global__ void k_wall_torque_final(int32_t n_inst, const InstDev* __restrict__ 
   const int lane = threadIdx.x;
   const InstDev& P = inst[k];
   double T[3] = {0.0, 0.0, 0.0};
+#pragma unroll 4
   for (int64_t c = lane; c < P.n_chunks; c += 32)
     for (int a = 0; a < 3; ++a) T[a] += partials[(P.chunk_base + c) * 3 + a];
   for (int o = 16; o > 0; o >>= 1)

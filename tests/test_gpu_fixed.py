@@ -88,3 +88,23 @@ def test_wall_torque_and_options_share_the_lists():
     assert np.abs(np.subtract(da["T_wall"], db["T_wall"])).max() <= 1e-11 * tw
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("partner", [(21.0, 40), (36.0, 70)])
+def test_lane_counts_give_the_same_bits(partner):
+    """The lanes that share a list (eight below 2^15 particles in all, four
+    below 2^18, then two) and the partition's tiles change no bit: a small
+    vessel alone and batched with one that takes the batch past each bound."""
+    a = synth.cylinder(6.3, 11, Omega=0.13, f_v=0.4, seed=9)
+    b = synth.cylinder(*partner, Omega=0.1, f_v=0.3, seed=10)
+    assert a.n < 1 << 15 and (1 << 15 < a.n + b.n < 1 << 18 or a.n + b.n > 1 << 18)
+    solo, both = sim_of(a), sim_of([a, b])
+    solo.step(2)
+    both.step(2)
+    x, y = solo.state_arrays(), both.state_arrays()
+    for k in x:
+        assert np.array_equal(x[k], y[k][:a.n]), k
+    dx, dy = solo.diagnostics(), both.diagnostics(0)
+    assert dx["T_wall"] == dy["T_wall"] and dx["L_orb"] == dy["L_orb"]
+    solo.close()
+    both.close()
