@@ -203,7 +203,7 @@ struct CellWs {
 
 // Neighbour sets.  The neighbour search writes, for every grid cell, its
 // candidate table: the particles of the 27-cell stencil in candidate order
-// (rows dz, dy, cells kc, sorted index), at most kMaxCand entries, each the
+// (cells in the search's stencil order, sorted index), at most kMaxCand entries, each the
 // candidate's sorted index in the low 26 bits and, in the top 6 bits, the
 // cell displacement code (dx+1) | (dy+1) << 2 | (dz+1) << 4 of the particle's
 // cell relative to the candidate's (used by the mixed form).  Per particle it
@@ -367,6 +367,25 @@ struct MaskWalk {
   }
 };
 
+// A list group of 8 entries (32 bytes, aligned) in one 256-bit load through
+// the read-only path, and in one store: a warp's groups are 1 KB contiguous,
+// 8 lines an access, where two 128-bit accesses touch them twice (the L1's
+// line lookups bound the mixed form's passes).
+__device__ __forceinline__ void ld_group(const uint32_t* p, uint32_t (&e)[8]) {
+  asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3]), "=r"(e[4]), "=r"(e[5]), "=r"(e[6]),
+        "=r"(e[7])
+      : "l"(p));
+}
+__device__ __forceinline__ void st_group(uint32_t* p, uint32_t a, uint32_t b, uint32_t c,
+                                         uint32_t d, uint32_t e, uint32_t f, uint32_t g,
+                                         uint32_t h) {
+  asm volatile("st.global.v8.u32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               :
+               : "l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h)
+               : "memory");
+}
+
 // Per-thread neighbour-list builder.  push() stores an entry in the thread's
 // shared-memory staging and advances the fill only if it is kept (a
 // predicated store, no branch); drain(), called whenever 32 or more entries
@@ -394,10 +413,9 @@ struct ListWriter {
   }
   __device__ __forceinline__ void write_group(uint32_t from) {
     if (written < groups) {
-      uint4* dst = reinterpret_cast<uint4*>(list + nbr_slot(n, i, written << 3));
       const uint32_t* q = st + from * stride;
-      dst[0] = make_uint4(q[0], q[stride], q[2 * stride], q[3 * stride]);
-      dst[1] = make_uint4(q[4 * stride], q[5 * stride], q[6 * stride], q[7 * stride]);
+      st_group(list + nbr_slot(n, i, written << 3), q[0], q[stride], q[2 * stride],
+               q[3 * stride], q[4 * stride], q[5 * stride], q[6 * stride], q[7 * stride]);
     }
     ++written;
   }

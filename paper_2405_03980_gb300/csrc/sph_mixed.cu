@@ -108,22 +108,39 @@ __device__ __forceinline__ bool normalize(float& o, int& c, float L, int lo, int
 // entry (whose top bits carry c_i - c_j + 1 per axis) and the two offsets;
 // exactly antisymmetric, and bit-identical to the candidate test that wrote
 // the entry.  The unit displacement d of an axis is decoded on the integer
-// and FP32 pipes without a table: the float with the bits of 2^23 + (d + 1)
-// is exactly 2^23 + d + 1, and subtracting 2^23 + 1 leaves d exactly.
-// d L is exact, so the fused multiply-add gives the same bits as the
-// candidate test's (c_i - c_j) L + (o_i - o_j).  (A 64-entry table of unit
-// displacements in shared memory cost more: its bank-conflicted lookups
-// shared the L1 data path with the neighbour gathers.)
-__device__ __forceinline__ float unit_disp(uint32_t code, int axis) {
-  return __int_as_float(0x4B000000 | ((code >> (2 * axis)) & 3u)) - 8388609.0f;
+// and FP32 pipes without a table: the float with the bits of 2^23 + k (d + 1),
+// k = 1, 4, 16 where the axis' two bits stand, is exactly that, and
+// subtracting 2^23 + k leaves k d exactly.  k d (L / k) is exact (k a power of
+// two), so the fused multiply-add gives the same bits as the candidate test's
+// (c_i - c_j) L + (o_i - o_j).  (A 64-entry table of unit displacements in
+// shared memory cost more: its bank-conflicted lookups shared the L1 data
+// path with the neighbour gathers.)
+__device__ __forceinline__ float disp_x(uint32_t c) {
+  return __int_as_float(0x4B000000 | (c & 3u)) - 8388609.0f;
+}
+__device__ __forceinline__ float disp_y4(uint32_t c) {
+  return __int_as_float(0x4B000000 | (c & 12u)) - 8388612.0f;
+}
+__device__ __forceinline__ float disp_z16(uint32_t c) {
+  return __int_as_float(0x4B000000 | (c & 48u)) - 8388624.0f;
 }
 
 __device__ __forceinline__ void entry_vec(const InstDev& P, uint32_t ent, const float4& oi,
                                           const float4& oj, float& dx, float& dy, float& dz) {
   const uint32_t c = ent >> kNbrIndexBits;
-  dx = fmaf(unit_disp(c, 0), P.cellf[0], oi.x - oj.x);
-  dy = fmaf(unit_disp(c, 1), P.cellf[1], oi.y - oj.y);
-  dz = fmaf(unit_disp(c, 2), P.cellf[2], oi.z - oj.z);
+  dx = fmaf(disp_x(c), P.cellf[0], oi.x - oj.x);
+  dy = fmaf(disp_y4(c), 0.25f * P.cellf[1], oi.y - oj.y);
+  dz = fmaf(disp_z16(c), 0.0625f * P.cellf[2], oi.z - oj.z);
+}
+
+// 1 / sqrt(x) for a normal x: the hardware estimate that rsqrtf is, without
+// its scaling of subnormal arguments (in the density, where a distance below
+// 1e-19 may read as 0: W is flat there; the pair pass keeps rsqrtf).
+constexpr float kMinR2 = 1.17549435e-38f;
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // The velocity and spin records of neighbour j: its 32-byte record in one
@@ -428,9 +445,8 @@ k_skin_list_mixed(int64_t n, MixBuf b, const InstDev* __restrict__ inst,
       uint32_t e[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
       for (uint32_t m, g = 0; (m = mk.next(e)) != 0u; ++g) {
         if (g < groups) {
-          uint4* dst = reinterpret_cast<uint4*>(nw.skin + nbr_slot(n, i, g << 3));
-          dst[0] = make_uint4(e[0], e[1], e[2], e[3]);
-          dst[1] = make_uint4(e[4], e[5], e[6], e[7]);
+          st_group(nw.skin + nbr_slot(n, i, g << 3), e[0], e[1], e[2], e[3], e[4], e[5], e[6],
+                   e[7]);
         }
         cnt += m;
       }
@@ -463,9 +479,9 @@ struct ShapedListWriter : ListWriter {
     if (written < groups) {
       const int64_t slot = nbr_slot(n, i, written << 3);
       const float* r = sw + from * stride;
-      float4* dw = reinterpret_cast<float4*>(wl + slot);
-      dw[0] = make_float4(r[0], r[stride], r[2 * stride], r[3 * stride]);
-      dw[1] = make_float4(r[4 * stride], r[5 * stride], r[6 * stride], r[7 * stride]);
+      const auto u = [&](uint32_t q) { return __float_as_uint(r[q * stride]); };
+      st_group(reinterpret_cast<uint32_t*>(wl + slot), u(0), u(1), u(2), u(3), u(4), u(5), u(6),
+               u(7));
     }
     ListWriter::write_group(from);
   }
@@ -540,11 +556,9 @@ k_density_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
     const float mrD0 = P.mr_f[0] * P.aD_f, mrD1 = P.mr_f[1] * P.aD_f;
     const float cut2 = P.cut2_f;
     const uint32_t scnt = checked_count(nw.skin_count[i], nw.skin_cap, err);
-    const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(nw.skin);
     for (uint32_t t0 = 0; t0 < scnt; t0 += 8) {
-      const int64_t g = 2 * ((int64_t)(t0 >> 3) * n + i);
-      const uint4 ga = groups[g], gb = groups[g + 1];
-      const uint32_t e[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+      uint32_t e[8];
+      ld_group(nw.skin + nbr_slot(n, i, t0), e);
       const uint32_t m = scnt - t0 < 8u ? scnt - t0 : 8u;
       float4 o[8];
 #pragma unroll
@@ -560,7 +574,7 @@ k_density_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
           if constexpr (!kFilter) out.push(e[u], keep);
           if (keep) {
             // r = r2 / sqrt(r2) from the approximate reciprocal square root
-            const float r = r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
+            const float r = r2 >= kMinR2 ? r2 * rsqrt_normal(r2) : 0.f;
             // (m_j / rho0) W(r) = (m_j aD / rho0) t^4 (2q + 1), t = 1 - q/2
             const float t1 = fmaf(-half_inv_h, r, 1.f);
             const float t2 = t1 * t1;
@@ -613,14 +627,10 @@ k_pfilter_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
   const float2 own = f.vp[i];
   Kahan num{own.x * own.y, 0.f}, den{own.x, 0.f};  // self term, W(0) / aD = 1
   const uint32_t cnt = checked_count(nw.count[i], nw.cap, err);
-  const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(nw.list);
-  const float4* __restrict__ shapes = reinterpret_cast<const float4*>(nw.wsh_f);
   for (uint32_t t0 = 0; t0 < cnt; t0 += 8) {
-    const int64_t g = 2 * ((int64_t)(t0 >> 3) * n + i);
-    const uint4 ga = groups[g], gb = groups[g + 1];
-    const float4 wa = shapes[g], wb = shapes[g + 1];
-    const uint32_t e[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-    const float ws[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+    uint32_t e[8], ws[8];
+    ld_group(nw.list + nbr_slot(n, i, t0), e);
+    ld_group(reinterpret_cast<const uint32_t*>(nw.wsh_f) + nbr_slot(n, i, t0), ws);
     const uint32_t m = cnt - t0 < 8u ? cnt - t0 : 8u;
     float2 vj[8];
 #pragma unroll
@@ -630,7 +640,7 @@ k_pfilter_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
 #pragma unroll
     for (uint32_t u = 0; u < 8; ++u) {
       if (u < m) {
-        const float w = vj[u].x * ws[u];
+        const float w = vj[u].x * __uint_as_float(ws[u]);
         gn += w * vj[u].y;
         gd += w;
       }
@@ -647,12 +657,29 @@ k_pfilter_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
 
 // ------------------------------------------------------------------ pair pass
 
-// The pair pass with the optional terms, one neighbour per step.  kOpt:
-// kOptLiteral if some instance uses the literal F_sn (coefficient of v_ij),
-// kOptCollision if some instance uses the collision model.  (The default
-// form, with neither, runs k_forces_mixed_x2 below.)
+// The pair pass with two neighbours of particle i per step, their FP32
+// arithmetic in packed pairs (f32x2: one instruction, two independent
+// operations each rounded as its scalar form).  Every pair scalar is formed
+// in an order independent of (i, j), so f_ji == -f_ij bit for bit.  A
+// neighbour slot past the list's end, or a coincident particle (r = 0:
+// density only), is evaluated on stand-in values and masked out.  The five
+// terms are collected along r_ij, u_ij and (literal F_sn) v_ij: shear
+// -A VV F dv/r^2 r_ij; rotational -B VV F u_ij + B VV F dv/r^2 r_ij
+// (r_ij . u_ij = r_ij . v_ij: the spin part of u_ij is normal to r_ij).
+// kOpt: kOptLiteral if some instance uses the literal F_sn (coefficient of
+// v_ij), kOptCollision if some instance uses the collision model.
+// The packed form wants 140 registers (160 with the options); bounding them
+// at 128 keeps 16 warps per SM at the cost of a few spilled loop constants
+// (with 12 warps the pass waits on its gathers: 1.08 against 1.02 ms with
+// collisions at 2.5M particles).  A pass of one neighbour per step took
+// 1.09 ms there (filter and collision model), 8 scalar operations where the
+// packed form issues 4.  The next group of entries is loaded after this
+// one's first pair (before it, 4 % slower: eight more live registers).  Bound
+// by the line lookups of the neighbour gathers (about 37 lines per
+// neighbour of a warp) and by issue: 7.30 -> 7.15 ms at 20.1M with the
+// 256-bit list loads and the decode of entry_vec.
 template <int BLOCK, int kOpt>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
 k_forces_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ inst, NbrWs nw,
                uint32_t* err) {
   const int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
@@ -678,7 +705,7 @@ k_forces_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ ins
   const float kA = (fl & SPH_TERM_SH) ? P.A_f : 0.f;
   const float kB = (fl & SPH_TERM_ROT) ? P.B_f : 0.f;
   const float kN = (fl & SPH_TERM_SN) ? P.C_l_f : 0.f;
-  const float hz = (fl & SPH_HPROJ) ? 0.f : 1.f;
+  const bool hproj = (fl & SPH_HPROJ) != 0;
   const bool lit = (kOpt & kOptLiteral) && (fl & SPH_SN_LITERAL) != 0;
   // collision model: col_dist^2 (0 when off); its coefficient
   // -(1 + e) mu_ij / dt is read, for the rare colliding pair only, from the
@@ -688,186 +715,9 @@ k_forces_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ ins
   // The species factors of the pair terms depend on j only through whether
   // j is inviscid (suffix 0) or not (suffix 1): mX = 1 for unlike species
   // (interfacial force, F_sn), mV = 1 for two viscous particles (shear,
-  // rotational); walls count as viscous.
-  const float mX0 = inv_i ? 0.f : 1.f;  // j inviscid
-  const float mX1 = inv_i ? 1.f : 0.f;  // j viscous or wall
-  const float mV1 = inv_i ? 0.f : 1.f;  // (mV = 0 for an inviscid j)
-  // The kernel constants cF (in F) and aD (in W) are folded in here, so
-  // that the pair loop forms only the shapes t^3 and t^4 (2q + 1).
-  const float cF = P.cF_f, aD = P.aD_f;
-  const float cP0 = kP * (m_i * P.m_f[0]) * cF, cP1 = kP * (m_i * P.m_f[1]) * cF;
-  const float cT0 = kT * mX0 * cF, cT1 = kT * mX1 * cF;
-  const float cBA1 = mV1 != 0.f ? (kB - kA) * cF : 0.f;
-  const float cB0 = -kB * 0.f, cB1 = -kB * mV1 * cF;
-  const float cN0 = -kN * mX0 * aD, cN1 = -kN * mX1 * aD;
-  const bool hproj = hz == 0.f;
-  const float half_inv_h = 0.5f * P.inv_h_f, two_inv_h = 2.f * P.inv_h_f;
-  const float hwx = 0.5f * wi.x, hwy = 0.5f * wi.y, hwz = 0.5f * wi.z;
-  // absolute position of i about the rotation axis (wall torque only)
-  const double xi = P.lo[0] + (double)cell_x(ci) * P.cell[0] + (double)oi.x;
-  const double yi = P.lo[1] + (double)cell_y(ci) * P.cell[1] + (double)oi.y;
-  const double zi = fold_z(P, P.lo[2] + (double)cell_z(ci) * P.cell[2] + (double)oi.z);
-  const float pxi = (float)xi, pyi = (float)yi, pzi = (float)zi;
-  // compensated sums across groups of 8 neighbours, plain FP32 sums inside
-  // a group
-  Kahan fx{0.f, 0.f}, fy{0.f, 0.f}, fz{0.f, 0.f}, tx{0.f, 0.f}, ty{0.f, 0.f}, tz{0.f, 0.f};
-  float gfx = 0.f, gfy = 0.f, gfz = 0.f, gtx = 0.f, gty = 0.f, gtz = 0.f;
-  float wx = 0.f, wy = 0.f, wz = 0.f;
-  const uint32_t cnt = checked_count(nw.count[i], nw.cap, err);
-  // The list is read one group of 8 entries (one 32-byte sector) at a time,
-  // the next group while the current one is evaluated; the neighbour record
-  // of the next entry is loaded one pair ahead.
-  const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(nw.list);
-  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  uint4 ga = make_uint4(0u, 0u, 0u, 0u), gb = ga;
-  float4 oj_n = zero4, vj_n = zero4, wj_n = zero4;
-  if (cnt > 0) {
-    ga = groups[2 * i];
-    gb = groups[2 * i + 1];
-    const uint32_t j0 = checked_index(ga.x & kNbrIndexMask, n, err);
-    oj_n = b.off[j0];
-    load_vs(b, j0, vj_n, wj_n);
-  }
-  for (uint32_t t0 = 0; t0 < cnt; t0 += 8) {
-    const uint32_t e[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-    if (t0 + 8 < cnt) {
-      const int64_t g = 2 * ((int64_t)((t0 >> 3) + 1) * n + i);
-      ga = groups[g];
-      gb = groups[g + 1];
-    }
-    const uint32_t m = cnt - t0 < 8u ? cnt - t0 : 8u;
-#pragma unroll
-    for (uint32_t u = 0; u < 8; ++u) {
-      if (u >= m) break;
-      const uint32_t ent = e[u];
-      const float4 oj = oj_n, vj = vj_n, wj = wj_n;
-      if (t0 + u + 1 < cnt) {
-        const uint32_t jn = checked_index((u < 7 ? e[u + 1] : ga.x) & kNbrIndexMask, n, err);
-        oj_n = b.off[jn];
-        load_vs(b, jn, vj_n, wj_n);
-      }
-      float dx, dy, dz;
-      entry_vec(P, ent, oi, oj, dx, dy, dz);
-      const float r2 = dx * dx + dy * dy + dz * dz;
-      if (!(r2 > 0.f)) continue;  // coincident particles: density only
-      const float inv_r = rsqrtf(r2);
-      const float r = r2 * inv_r;
-      const float inv_r2 = inv_r * inv_r;
-      const float t1 = fmaf(-half_inv_h, r, 1.f);         // 1 - q/2
-      const float t2 = t1 * t1;
-      const float F = t2 * t1;                            // F / cF
-      const float W = (t2 * t2) * fmaf(two_inv_h, r, 1.f);  // W / aD
-      const bool vis_j = oj.w != 0.f;
-      // symmetric pair scalars (products taken in an order independent of i, j)
-      const float VV = vi.w * vj.w;
-      const float vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
-      // half the spin sum, (w_i + w_j) / 2, the same bits from either side
-      const float sx = fmaf(0.5f, wj.x, hwx), sy = fmaf(0.5f, wj.y, hwy),
-                  sz = fmaf(0.5f, wj.z, hwz);
-      const float ux = fmaf(dy, sz, fmaf(-dz, sy, vx));
-      const float uy = fmaf(dz, sx, fmaf(-dx, sz, vy));
-      const float uz = fmaf(dx, sy, fmaf(-dy, sx, vz));
-      const float dv = dx * vx + dy * vy + dz * vz;  // r_ij . v_ij (symmetric)
-      // the five terms collected along r_ij, u_ij and (literal F_sn) v_ij:
-      // shear -A VV F dv/r^2 r_ij; rotational -B VV F u_ij + B VV F dv/r^2 r_ij
-      // (r_ij . u_ij = r_ij . v_ij: the spin part of u_ij is normal to r_ij)
-      const float VF = VV * F;
-      const float aP = (vis_j ? cP1 : cP0) * ((wi.w + wj.w) * F);
-      const float aT = (vis_j ? cT1 : cT0) * VF;
-      const float aV = (VF * inv_r2) * ((vis_j ? cBA1 : 0.f) * dv);
-      const float bR = (vis_j ? cB1 : cB0) * VF;
-      const float bN = (vis_j ? cN1 : cN0) * (VV * W);
-      float base = aP + aV;  // the z component drops aT under the projection
-      // collision of an approaching pair closer than col_dist: the central
-      // force m_i dv_i / dt = -(1 + e) mu_ij (r_ij . v_ij) / (r^2 dt) r_ij
-      if ((kOpt & kOptCollision) && r2 < col2 && dv < 0.f)
-        base += P.cC_f[si + (vis_j ? 1 : 0)] * (dv * inv_r2);
-      const float al = base + aT;
-      const float alz = hproj ? base : al;
-      const float bu = lit ? bR : bR + bN;
-      float pfx = al * dx + bu * ux;
-      float pfy = al * dy + bu * uy;
-      float pfz = alz * dz + bu * uz;
-      if ((kOpt & kOptLiteral) && lit) {
-        pfx += bN * vx;
-        pfy += bN * vy;
-        pfz += bN * vz;
-      }
-      gfx += pfx;
-      gfy += pfy;
-      gfz += pfz;
-      // spin torque -1/2 r_ij x (f_rot + f_sn) = -1/2 bu (r_ij x u_ij); the
-      // factor -1/2 (exact) is applied to the sums
-      const float qx = bu * (dy * uz - dz * uy);
-      const float qy = bu * (dz * ux - dx * uz);
-      const float qz = bu * (dx * uy - dy * ux);
-      gtx += qx;
-      gty += qy;
-      gtz += qz;
-      if (oj.w >= 2.f) {
-        wx += fmaf(-0.5f, qx, pyi * pfz - pzi * pfy);
-        wy += fmaf(-0.5f, qy, pzi * pfx - pxi * pfz);
-        wz += fmaf(-0.5f, qz, pxi * pfy - pyi * pfx);
-      }
-    }
-    fx.add(gfx);
-    fy.add(gfy);
-    fz.add(gfz);
-    tx.add(gtx);
-    ty.add(gty);
-    tz.add(gtz);
-    gfx = gfy = gfz = gtx = gty = gtz = 0.f;
-  }
-  const float inv_m = P.inv_m_f[si], inv_I = P.inv_I_f[si];
-  const float ax = fx.value(), ay = fy.value(), az = fz.value();
-  const float bx = -0.5f * tx.value(), by = -0.5f * ty.value(), bz = -0.5f * tz.value();
-  f.acc[i] = make_float4(ax * inv_m, ay * inv_m, az * inv_m, 0.f);
-  f.dspin[i] = make_float4(bx * inv_I, by * inv_I, bz * inv_I, 0.f);
-  f.tw[i] = make_float4(wx, wy, wz, 0.f);
-  if (!finite3f(ax, ay, az) || !finite3f(bx, by, bz)) latch(err, ERR_NONFINITE);
-}
-
-// The pair pass of the default form (neither the literal F_sn nor the
-// collision model) with two neighbours of particle i per step, their FP32
-// arithmetic in packed pairs (f32x2: one instruction, two independent
-// operations each rounded as its scalar form), where the thread-per-pair
-// loop above issues one instruction per operation.  Every pair scalar is
-// formed in an order independent of (i, j) as there, so f_ji == -f_ij bit
-// for bit.  A neighbour slot past the list's end, or a coincident particle
-// (r = 0: density only), is evaluated on stand-in values and masked out.
-// The packed form wants more registers (140) than the scalar loop; bounding
-// them at 128 keeps the scalar loop's 16 warps per SM at the cost of a few
-// spilled loop constants (with 12 warps the pass waited on its gathers).
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
-k_forces_mixed_x2(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ inst, NbrWs nw,
-                  uint32_t* err) {
-  const int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x;
-  if (i >= n) return;
-  const float4 oi = b.off[i];
-  const int sp_i = (int)oi.w;
-  if (sp_i >= 2) {
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    f.acc[i] = z;
-    f.dspin[i] = z;
-    f.tw[i] = z;
-    return;
-  }
-  const InstDev& P = inst[b.inst[i]];
-  const uint32_t ci = b.cell[i];
-  float4 vi, wi;  // w: V_i and P_i / rho_i^2
-  load_vs(b, i, vi, wi);
-  const int si = sp_i == 0 ? 0 : 1;
-  const float m_i = P.m_f[si];
-  const uint32_t fl = P.flags;
-  const float kP = (fl & SPH_TERM_P) ? 1.f : 0.f;
-  const float kT = (fl & SPH_TERM_T) ? P.C_T_f : 0.f;
-  const float kA = (fl & SPH_TERM_SH) ? P.A_f : 0.f;
-  const float kB = (fl & SPH_TERM_ROT) ? P.B_f : 0.f;
-  const float kN = (fl & SPH_TERM_SN) ? P.C_l_f : 0.f;
-  const bool hproj = (fl & SPH_HPROJ) != 0;
-  const bool inv_i = sp_i == 0;
-  // species factors and kernel constants as in k_forces_mixed
+  // rotational); walls count as viscous.  The kernel constants cF (in F) and
+  // aD (in W) are folded in, so that the loop forms only the shapes t^3 and
+  // t^4 (2q + 1).
   const float mX0 = inv_i ? 0.f : 1.f, mX1 = inv_i ? 1.f : 0.f, mV1 = inv_i ? 0.f : 1.f;
   const float cF = P.cF_f, aD = P.aD_f;
   const float cP0 = kP * (m_i * P.m_f[0]) * cF, cP1 = kP * (m_i * P.m_f[1]) * cF;
@@ -882,17 +732,17 @@ k_forces_mixed_x2(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ 
   // packed constants; the differences with i's own records are formed as two
   // scalar operations each (the same roundings), which keeps those records
   // out of packed registers and the kernel within its register bound
-  const f2 LX = f2_splat(P.cellf[0]), LY = f2_splat(P.cellf[1]), LZ = f2_splat(P.cellf[2]);
-  const f2 ONE = f2_splat(1.f), MAGIC = f2_splat(8388609.0f);
+  const f2 LX = f2_splat(P.cellf[0]), LY = f2_splat(0.25f * P.cellf[1]),
+           LZ = f2_splat(0.0625f * P.cellf[2]);
+  const f2 ONE = f2_splat(1.f);
   const f2 NHIH = f2_splat(-0.5f * P.inv_h_f), TIH = f2_splat(2.f * P.inv_h_f);
   const float hwx = 0.5f * wi.x, hwy = 0.5f * wi.y, hwz = 0.5f * wi.z;
   Kahan fx{0.f, 0.f}, fy{0.f, 0.f}, fz{0.f, 0.f}, tx{0.f, 0.f}, ty{0.f, 0.f}, tz{0.f, 0.f};
   float wx = 0.f, wy = 0.f, wz = 0.f;
   const uint32_t cnt = checked_count(nw.count[i], nw.cap, err);
-  const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(nw.list);
   // records of the next two entries, loaded one step ahead; a slot past the
   // list's end takes the first entry's records
-  uint4 ga = make_uint4(0u, 0u, 0u, 0u), gb = ga;
+  uint32_t ge[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};  // the next group
   float4 oa_n, va_n, wa_n, ob_n, vb_n, wb_n;
   auto fetch2 = [&](uint32_t ea, uint32_t eb, bool has_b) {
     const uint32_t ja = checked_index(ea & kNbrIndexMask, n, err);
@@ -903,17 +753,13 @@ k_forces_mixed_x2(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ 
     load_vs(b, jb, vb_n, wb_n);
   };
   if (cnt > 0) {
-    ga = groups[2 * i];
-    gb = groups[2 * i + 1];
-    fetch2(ga.x, ga.y, cnt > 1);
+    ld_group(nw.list + nbr_slot(n, i, 0), ge);
+    fetch2(ge[0], ge[1], cnt > 1);
   }
   for (uint32_t t0 = 0; t0 < cnt; t0 += 8) {
-    const uint32_t e[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-    if (t0 + 8 < cnt) {
-      const int64_t gi = 2 * ((int64_t)((t0 >> 3) + 1) * n + i);
-      ga = groups[gi];
-      gb = groups[gi + 1];
-    }
+    uint32_t e[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) e[u] = ge[u];
     const uint32_t m = cnt - t0 < 8u ? cnt - t0 : 8u;
     f2 GFX = 0ull, GFY = 0ull, GFZ = 0ull, GTX = 0ull, GTY = 0ull, GTZ = 0ull;
 #pragma unroll
@@ -922,20 +768,17 @@ k_forces_mixed_x2(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ 
       const bool has_b = u + 1 < m;
       const uint32_t ea = e[u], eb = has_b ? e[u + 1] : e[u];
       const float4 oa = oa_n, va = va_n, wa = wa_n, ob = ob_n, vb = vb_n, wb = wb_n;
+      if (u == 2 && t0 + 8 < cnt) ld_group(nw.list + nbr_slot(n, i, t0 + 8), ge);
       if (t0 + u + 2 < cnt) {
-        const uint32_t na = u < 6 ? e[u + 2] : ga.x;
-        const uint32_t nb = u < 6 ? e[u + 3] : ga.y;
+        const uint32_t na = u < 6 ? e[u + 2] : ge[0];
+        const uint32_t nb = u < 6 ? e[u + 3] : ge[1];
         fetch2(na, nb, t0 + u + 3 < cnt);
       }
       // pair vectors (c_i - c_j) L + (o_i - o_j), the unit displacement of
       // each axis decoded as in entry_vec
       const uint32_t ca = ea >> kNbrIndexBits, cb = eb >> kNbrIndexBits;
-      const f2 EX = f2_sub(f2_make(__int_as_float(0x4B000000 | (ca & 3u)),
-                                   __int_as_float(0x4B000000 | (cb & 3u))), MAGIC);
-      const f2 EY = f2_sub(f2_make(__int_as_float(0x4B000000 | ((ca >> 2) & 3u)),
-                                   __int_as_float(0x4B000000 | ((cb >> 2) & 3u))), MAGIC);
-      const f2 EZ = f2_sub(f2_make(__int_as_float(0x4B000000 | (ca >> 4)),
-                                   __int_as_float(0x4B000000 | (cb >> 4))), MAGIC);
+      const f2 EX = f2_make(disp_x(ca), disp_x(cb)), EY = f2_make(disp_y4(ca), disp_y4(cb)),
+               EZ = f2_make(disp_z16(ca), disp_z16(cb));
       const f2 dX = f2_fma(EX, LX, f2_make(oi.x - oa.x, oi.x - ob.x));
       const f2 dY = f2_fma(EY, LY, f2_make(oi.y - oa.y, oi.y - ob.y));
       const f2 dZ = f2_fma(EZ, LZ, f2_make(oi.z - oa.z, oi.z - ob.z));
@@ -975,13 +818,36 @@ k_forces_mixed_x2(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ 
       const f2 bR = f2_mul(f2_make(visa ? cB1 : cB0, visb ? cB1 : cB0), VF);
       const f2 bN = f2_mul(f2_make(visa ? cN1 : cN0, visb ? cN1 : cN0), f2_mul(VV, W));
       const f2 MK = f2_make(oka ? 1.f : 0.f, okb ? 1.f : 0.f);
-      const f2 base = f2_add(aP, aV);
+      f2 base = f2_add(aP, aV);
+      if (kOpt & kOptCollision) {
+        // collision of an approaching pair closer than col_dist: the central
+        // force m_i dv_i / dt = -(1 + e) mu_ij (r_ij . v_ij) / (r^2 dt) r_ij
+        // (its test on r^2 in the scalar order of operations)
+        float dva, dvb;
+        f2_split(DV, dva, dvb);
+        float xa, xb, ya, yb, za, zb;
+        f2_split(dX, xa, xb);
+        f2_split(dY, ya, yb);
+        f2_split(dZ, za, zb);
+        const bool hita = xa * xa + ya * ya + za * za < col2 && dva < 0.f;
+        const bool hitb = xb * xb + yb * yb + zb * zb < col2 && dvb < 0.f;
+        if (hita || hitb)
+          base = f2_add(base, f2_mul(f2_make(hita ? P.cC_f[si + (visa ? 1 : 0)] : 0.f,
+                                             hitb ? P.cC_f[si + (visb ? 1 : 0)] : 0.f),
+                                     f2_mul(DV, IR2)));
+      }
       const f2 AL = f2_mul(f2_add(base, aT), MK);
       const f2 ALZ = hproj ? f2_mul(base, MK) : AL;
-      const f2 BU = f2_mul(f2_add(bR, bN), MK);
-      const f2 pX = f2_fma(AL, dX, f2_mul(BU, uX));
-      const f2 pY = f2_fma(AL, dY, f2_mul(BU, uY));
-      const f2 pZ = f2_fma(ALZ, dZ, f2_mul(BU, uZ));
+      const f2 BU = f2_mul(((kOpt & kOptLiteral) && lit) ? bR : f2_add(bR, bN), MK);
+      f2 pX = f2_fma(AL, dX, f2_mul(BU, uX));
+      f2 pY = f2_fma(AL, dY, f2_mul(BU, uY));
+      f2 pZ = f2_fma(ALZ, dZ, f2_mul(BU, uZ));
+      if ((kOpt & kOptLiteral) && lit) {  // F_sn along v_ij
+        const f2 BN = f2_mul(bN, MK);
+        pX = f2_fma(BN, vX, pX);
+        pY = f2_fma(BN, vY, pY);
+        pZ = f2_fma(BN, vZ, pZ);
+      }
       GFX = f2_add(GFX, pX);
       GFY = f2_add(GFY, pY);
       GFZ = f2_add(GFZ, pZ);
@@ -1200,16 +1066,6 @@ cudaError_t launch_forces_mixed(int64_t n, const MixBuf& b, const MixFields& f,
                  g64 = (unsigned)((n + 63) / 64);
   // the pair pass carries only the options some instance uses
   const int opt = (lc.any_literal ? kOptLiteral : 0) | (lc.any_collision ? kOptCollision : 0);
-  if (opt == 0) {  // the default form: two neighbours per step in packed FP32
-    if (lc.block_forces == 256)
-      k_forces_mixed_x2<256><<<g256, 256, 0, s>>>(n, b, f, inst, nw, err);
-    else if (lc.block_forces == 64)
-      k_forces_mixed_x2<64><<<g64, 64, 0, s>>>(n, b, f, inst, nw, err);
-    else
-      k_forces_mixed_x2<128><<<g128, 128, 0, s>>>(n, b, f, inst, nw, err);
-    if (launches) ++*launches;
-    return cudaGetLastError();
-  }
   auto go = [&](auto kopt) {
     constexpr int O = decltype(kopt)::value;
     if (lc.block_forces == 256)
@@ -1219,7 +1075,9 @@ cudaError_t launch_forces_mixed(int64_t n, const MixBuf& b, const MixFields& f,
     else
       k_forces_mixed<128, O><<<g128, 128, 0, s>>>(n, b, f, inst, nw, err);
   };
-  if (opt == kOptCollision)
+  if (opt == 0)
+    go(std::integral_constant<int, 0>());
+  else if (opt == kOptCollision)
     go(std::integral_constant<int, kOptCollision>());
   else  // the literal F_sn, with or without collisions
     go(std::integral_constant<int, kOptLiteral | kOptCollision>());
