@@ -4,7 +4,7 @@
 // Every particle of a cell has the same 27-cell candidate set: the 9 rows
 // (dy, dz) of x-adjacent cells cx-1..cx+1, each row one contiguous run of the
 // sorted order per cell.  A warp takes one cell, writes its candidate
-// sequence (rows dz, dy, cells kc, index j) once as the cell's candidate
+// sequence (cells in the order kStencil, index j) once as the cell's candidate
 // table, and tests the candidates with the lanes spread over the CANDIDATES:
 // for each target particle t of the cell, the 32 lanes test 32 candidates at
 // once and a ballot gives the 32-bit hit mask of (t, chunk), so no lane idles
@@ -53,6 +53,21 @@ __device__ __forceinline__ void latch(uint32_t* err, uint32_t bit) {
   if ((*(volatile uint32_t*)err & bit) == 0u) atomicOr(err, bit);
 }
 
+// The cells (dz + 1) 9 + (dy + 1) 3 + kc of the 27-cell stencil in candidate
+// order: rows in opposite pairs, their cells in turn with x descending, the
+// cell's own row third.  The lanes of a warp walk their lists in step, and
+// share lines of the gathered records only while their walks stay at the same
+// place of the table.  A particle near one face of its cell has more
+// neighbours behind that face and fewer behind the opposite one, so with
+// opposite cells side by side the lengths even out every two cells; in the
+// order dz, dy, kc the walks drift apart over a whole plane of nine.  Counted
+// on rotated, jittered lattices, the density's and the pair pass's gathers
+// touch a third fewer lines.  At 20.1M particles, mixed form: density 5.56 ->
+// 5.19 ms, pair pass 7.19 -> 6.98, list builds 1.25 -> 1.08 ms a step; FP64
+// form at 2.5M: density 1.84 -> 1.78, pair pass 4.80 -> 4.75.
+__device__ const uint8_t kStencil[27] = {23, 5, 22, 4, 21, 3, 17, 11, 16, 10, 15, 9, 14, 13,
+                                         12, 26, 2, 25, 1, 24, 0, 20, 8, 19, 7, 18, 6};
+constexpr int kSelfRun = 13;  // the run of the cell itself
 // r^2 of a pair vector with an explicit rounding sequence, so that both
 // search mappings below classify every candidate with the same bits.
 __device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
@@ -71,6 +86,7 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
   const InstDev& P = inst[blockIdx.y];
   const int64_t ncells = (int64_t)P.nx * P.ny * P.nz;
   const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int sc = kStencil[lane < 27 ? lane : 0];  // this lane's cell of the stencil
   // the warps of a bounded grid take the instance's cells in turn, so that a
   // step whose gate is closed costs a few thousand empty blocks at most
   for (int64_t l = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < ncells;
@@ -83,11 +99,11 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
     const int cy = (int)((l / P.nx) % P.ny);
     const int cz = (int)(l / ((int64_t)P.nx * P.ny));
 
-    // run table: lane r < 27 holds run r = (dz + 1) 9 + (dy + 1) 3 + kc, the
-    // particles of cell (cx - 1 + kc, cy + dy, cz + dz)
+    // run table: lane r < 27 holds run r, the particles of the stencil's cell
+    // kStencil[r]: (cx - 1 + kc, cy + dy, cz + dz)
     uint32_t rj0 = 0, rlen = 0, rcode = 0;
     if (lane < 27) {
-      const int dz = lane / 9 - 1, dy = (lane / 3) % 3 - 1, kc = lane % 3;
+      const int dz = sc / 9 - 1, dy = (sc / 3) % 3 - 1, kc = sc % 3;
       int z2 = cz + dz;
       if (P.periodic_z) z2 = z2 < 0 ? z2 + P.nz : (z2 >= P.nz ? z2 - P.nz : z2);
       const int64_t key =
@@ -114,7 +130,7 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
     }
     if (lane == 0) nw.ncand[g] = total;
     uint32_t* __restrict__ table = nw.cand + g * kMaxCand;
-    const uint32_t pre_self = __shfl_sync(~0u, rpre, 13);  // the cell's own run
+    const uint32_t pre_self = __shfl_sync(~0u, rpre, kSelfRun);  // the cell's own run
     const float cut2 = P.skin_cut2_f;
 
     bool table_done = false;
@@ -220,22 +236,23 @@ k_cell_search(int64_t n, const float4* __restrict__ rec, const InstDev* __restri
   }
 }
 
-// FP64 form: the run of class c in stencil cell r of a cell, by lane r < 27,
-// as positions in the candidate sequence (inviscid candidates of all cells,
+// FP64 form: the run of class c in stencil cell r of a cell, sc = kStencil[r],
+// by lane r < 27, as positions in the candidate sequence (inviscid candidates of all cells,
 // then viscous, then walls).
 struct ClassRuns {
   uint32_t j0[3], len[3], pre[3];  // first sorted index, length, first position
   uint32_t end[3];                 // position after the class (the same in all lanes)
 };
 __device__ __forceinline__ ClassRuns class_runs(const InstDev& P, const CellWs& cw, int64_t n,
-                                                int cx, int cy, int cz, int lane, uint32_t* err) {
+                                                int cx, int cy, int cz, int lane, int sc,
+                                                uint32_t* err) {
   ClassRuns R;
   int64_t key = 0;
   if (lane < 27) {
-    int z2 = cz + lane / 9 - 1;
+    int z2 = cz + sc / 9 - 1;
     if (P.periodic_z) z2 = z2 < 0 ? z2 + P.nz : (z2 >= P.nz ? z2 - P.nz : z2);
-    key = P.cell_base + ((int64_t)(cx - 1 + lane % 3) +
-                         (int64_t)P.nx * ((cy + (lane / 3) % 3 - 1) + (int64_t)P.ny * z2)) *
+    key = P.cell_base + ((int64_t)(cx - 1 + sc % 3) +
+                         (int64_t)P.nx * ((cy + (sc / 3) % 3 - 1) + (int64_t)P.ny * z2)) *
                             P.slabs;
   }
   uint32_t base = 0;
@@ -278,6 +295,7 @@ k_cell_search64(int64_t n, const InstDev* __restrict__ inst, CellWs cw, NbrWs nw
   const InstDev& P = inst[blockIdx.y];
   const int64_t ncells = (int64_t)P.nx * P.ny * P.nz;
   const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int sc = kStencil[lane < 27 ? lane : 0];  // this lane's cell of the stencil
   for (int64_t l = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < ncells;
        l += wstride) {
     const int64_t key0 = P.cell_base + l * P.slabs;
@@ -286,8 +304,8 @@ k_cell_search64(int64_t n, const InstDev* __restrict__ inst, CellWs cw, NbrWs nw
     const int cx = (int)(l % P.nx);
     const int cy = (int)((l / P.nx) % P.ny);
     const int cz = (int)(l / ((int64_t)P.nx * P.ny));
-    const ClassRuns R = class_runs(P, cw, n, cx, cy, cz, lane, err);
-    const uint32_t rcode = run_code(lane);
+    const ClassRuns R = class_runs(P, cw, n, cx, cy, cz, lane, sc, err);
+    const uint32_t rcode = run_code(sc);
     const int64_t g = key0 / P.slabs;  // grid cell over all instances
     uint32_t total = R.end[2];
     if (total > (uint32_t)kMaxCand) {  // more candidates than the table holds
@@ -311,13 +329,14 @@ k_cell_search64(int64_t n, const InstDev* __restrict__ inst, CellWs cw, NbrWs nw
       sm.tz[lane] = mine.z;
       const bool active = lane < nt && mine.w != 3.f;  // outer-wall particles keep no list
       if (__ballot_sync(~0u, active) == 0u) continue;
-      // candidate position of i itself: in its class's run of stencil cell 13
+      // candidate position of i itself: in its class's run of its own cell
       const int ci = mine.w < 2.f ? (int)mine.w : 2;
       uint32_t self_q = ~0u;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const uint32_t p13 = __shfl_sync(~0u, R.pre[c], 13), j13 = __shfl_sync(~0u, R.j0[c], 13);
-        if (active && ci == c) self_q = p13 + (i - j13);
+        const uint32_t p = __shfl_sync(~0u, R.pre[c], kSelfRun);
+        const uint32_t j = __shfl_sync(~0u, R.j0[c], kSelfRun);
+        if (active && ci == c) self_q = p + (i - j);
       }
       for (uint32_t s0 = 0; s0 < total; s0 += kSeg) {
         const uint32_t nseg = min((uint32_t)kSeg, total - s0);
@@ -416,12 +435,13 @@ k_cell_search64_tpp(int64_t n, Fp64Buf b, const InstDev* __restrict__ inst, Cell
     bool over = false;
     for (int c = 0; c < 3; ++c) {
       for (int r = 0; r < 27 && !over; ++r) {
-        const int zu = cz + r / 9 - 1;  // unwrapped z cell of the run
+        const int sc = kStencil[r];
+        const int zu = cz + sc / 9 - 1;  // unwrapped z cell of the run
         int z2 = zu;
         if (P.periodic_z) z2 = z2 < 0 ? z2 + P.nz : (z2 >= P.nz ? z2 - P.nz : z2);
         const int64_t key = P.cell_base +
-                            ((int64_t)(cx - 1 + r % 3) +
-                             (int64_t)P.nx * ((cy + (r / 3) % 3 - 1) + (int64_t)P.ny * z2)) *
+                            ((int64_t)(cx - 1 + sc % 3) +
+                             (int64_t)P.nx * ((cy + (sc / 3) % 3 - 1) + (int64_t)P.ny * z2)) *
                                 P.slabs;
         const uint32_t j0 = cw.start[key + (c ? c + 1 : 0)];
         uint32_t len = cw.start[key + c + 2] - j0;
@@ -433,7 +453,7 @@ k_cell_search64_tpp(int64_t n, Fp64Buf b, const InstDev* __restrict__ inst, Cell
             break;
           }
           const uint32_t j = j0 + e;
-          if (writer) table[q] = j | run_code(r);
+          if (writer) table[q] = j | run_code(sc);
           if (active) {
             const float4 o = rec[j];
             if ((int64_t)j != i &&
@@ -492,7 +512,8 @@ k_cell_search_tpp(int64_t n, const float4* __restrict__ rec,
     uint32_t q = 0, word = 0, hits = 0, self_q = ~0u;
     bool over = false;
     for (int r = 0; r < 27 && !over; ++r) {
-      const int dz = r / 9 - 1, dy = (r / 3) % 3 - 1, kc = r % 3;
+      const int sc = kStencil[r];
+      const int dz = sc / 9 - 1, dy = (sc / 3) % 3 - 1, kc = sc % 3;
       int z2 = cz + dz;
       if (P.periodic_z) z2 = z2 < 0 ? z2 + P.nz : (z2 >= P.nz ? z2 - P.nz : z2);
       const int64_t key =
@@ -501,7 +522,7 @@ k_cell_search_tpp(int64_t n, const float4* __restrict__ rec,
       const uint32_t rj0 = cw.start[key];
       uint32_t rlen = cw.start[key + S] - rj0;
       if (!bounds_ok((int64_t)rj0 + rlen <= n, err)) rlen = 0;
-      if (r == 13) self_q = q + ((uint32_t)i - rj0);  // run 13 is the particle's own cell
+      if (r == kSelfRun) self_q = q + ((uint32_t)i - rj0);
       const uint32_t code = ((uint32_t)(2 - kc) | ((uint32_t)(1 - dy) << 2) |
                              ((uint32_t)(1 - dz) << 4)) << kNbrIndexBits;
       // (c_i - c_j) L per axis (exact): the run's cell is c_i + (kc - 1, dy, dz),
