@@ -521,16 +521,22 @@ __device__ __forceinline__ float pair_r2f(float dx, float dy, float dz) {
 // the entries of its reused list that lie within 2h now (r^2 < (2h)^2 on the
 // current offsets and the entry's cell-displacement code), which are also
 // written, in order, as the particle's neighbour list for the pair pass.
-// The list is read one 32-byte group of 8 entries at a time, and the 8
-// offset records are loaded together before the 8 pairs are tested.
+// The list is read one 32-byte group of 8 entries at a time, and its
+// offset records are loaded kAhead together, ahead of the pairs' tests.
+// Bound by the latency and the line lookups of these gathers: seven blocks of
+// 128 threads per SM (72 registers) take 4.89 ms at 20.1M particles where six
+// (80) took 5.19; eight (64) spill and take 7.9.  With six loads ahead the
+// filter's form fits in 72 registers too: 775 -> 752 us at 2.5M (all eight
+// ahead spill: 816); without the filter six ahead cost 2 % and four 7 %.
 // kFilter: some instance uses the pressure filter; the kernel shape of every
 // list entry is then stored beside the list (nw.wsh_f) for the filter, staged
 // with the entries and written with them as full sectors (drained at 16
 // entries, so that the two stagings take the shared memory of one).
 template <int BLOCK, bool kFilter>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, kFilter ? 0 : 7 * 128 / BLOCK)
 k_density_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ inst, NbrWs nw,
                 uint32_t* err) {
+  constexpr uint32_t kAhead = kFilter ? 6 : 8;
   constexpr int kDrain = kFilter ? 16 : kDrainAt;
   constexpr int kWords = kFilter ? 24 : kStageWords;
   static_assert(kWords >= kDrain - 1 + 8, "staging holds a drain's remainder and a batch");
@@ -561,11 +567,14 @@ k_density_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
       ld_group(nw.skin + nbr_slot(n, i, t0), e);
       const uint32_t m = scnt - t0 < 8u ? scnt - t0 : 8u;
       float4 o[8];
-#pragma unroll
-      for (uint32_t u = 0; u < 8; ++u)
+      const auto load = [&](uint32_t u) {
         if (u < m) o[u] = b.off[checked_index(e[u] & kNbrIndexMask, n, err)];
+      };
+#pragma unroll
+      for (uint32_t u = 0; u < kAhead; ++u) load(u);
 #pragma unroll
       for (uint32_t u = 0; u < 8; ++u) {
+        if (u + kAhead < 8) load(u + kAhead);
         if (u < m) {
           float dx, dy, dz;
           entry_vec(P, e[u], oi, o[u], dx, dy, dz);
