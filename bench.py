@@ -89,8 +89,8 @@ DENSITY_FLOPS_PER_PAIR = {"fp64": 18, "mixed": 29}
 # position record in, rho and P (and V, P/rho^2 for the pair pass) out.  Pair
 # pass: position, velocity, spin, V and P/rho^2 in, a and alpha out.
 ALGO_BYTES_PER_PARTICLE = {"k_density_mixed": 4 + 16 + 16, "k_density_fp64": 32 + 32,
-                           "k_forces_mixed": 4 + 48 + 32, "k_forces_mixed_x2": 4 + 48 + 32,
-                           "k_forces_fp64": 96 + 64}
+                           "k_forces_mixed": 4 + 48 + 32,
+                           "k_forces_fx": 96 + 64, "k_forces_fp64": 96 + 64}
 # Optional steps of Algorithm 1 (--extras).  The pressure filter streams each
 # fluid/inner-wall row's neighbour list and the kernel shapes the density
 # pass stored beside it (4 B + 4 B mixed, 4 B + 8 B FP64 per neighbour) and
@@ -649,9 +649,9 @@ def run_ours(args, dist):
         byc = FORCE_FLOPS_BY_CLASS[f]
         fl_forces = sum(byc[k] * cls[k] for k in cls) + (
             COLLISION_FLOPS_PER_PAIR * uq if "collision" in extras else 0)
-        # the mixed form's default pair pass takes two neighbours per step in
-        # packed FP32; with the collision model it runs the one-neighbour loop
-        fkern = ("k_forces_mixed_x2" if f == "mixed" and "collision" not in extras
+        # the FP64 form's pair pass forms its geometry and sums in fixed point on
+        # the integer pipe; with the collision model it runs in FP64 throughout
+        fkern = ("k_forces_fx" if f == "fp64" and "collision" not in extras
                  else f"k_forces_{f}")
         stages = [("forces", fkern, fl_forces / max(uq, 1), uq,
                    "unique pairs with a fluid particle (" +
@@ -664,7 +664,7 @@ def run_ours(args, dist):
         # the builds per step
         bps = results[f]["list_builds_per_step"]
         t = results[f]["stages"]["cell_search"] / (bps if bps > 0 else 1.0)
-        kern = f"k_cell_search<{str(f == 'mixed').lower()}>"
+        kern = "k_cell_search" if f == "mixed" else "k_cell_search64"
         by = SEARCH_ALGO_BYTES_PER_PARTICLE[f] * n_part
         ach = by / (t * 1e-3) / 1e9
         roofs.setdefault(f, {})["cell_search"] = {

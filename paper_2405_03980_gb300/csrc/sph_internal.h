@@ -203,8 +203,8 @@ struct CellWs {
 
 // Neighbour sets.  The neighbour search writes, for every grid cell, its
 // candidate table: the particles of the 27-cell stencil in candidate order
-// (cells in the search's stencil order, sorted index), at most kMaxCand entries, each the
-// candidate's sorted index in the low 26 bits and, in the top 6 bits, the
+// (cells in the search's stencil order, sorted index), at most kMaxCand
+// entries, each the candidate's sorted index in the low 26 bits and, in the top 6 bits, the
 // cell displacement code (dx+1) | (dy+1) << 2 | (dz+1) << 4 of the particle's
 // cell relative to the candidate's (used by the mixed form).  Per particle it
 // writes one bit per candidate of its cell: word k of particle i, at
@@ -241,10 +241,11 @@ struct NbrWs {
   uint32_t* count;      // neighbours per particle (list length)
   // FP64 form: a particle's list holds its inviscid neighbours, then the
   // viscous ones, then the walls, as the search's prefilter finds them; an
-  // entry that the density pass finds beyond 2h names the particle itself.  parts packs the entries of the first two classes (11 bits each)
-  // and the entries beyond 2h (10 bits).  Species partition of the fluid particles for
-  // the pair pass: order[0 .. n_inv) inviscid, then the viscous ones, each in
-  // sorted order.
+  // entry that the density pass finds beyond 2h names the particle itself.
+  // parts packs the entries of the first two classes (11 bits each) and the
+  // entries beyond 2h (10 bits).  Species partition of the fluid particles
+  // for the pair pass: order[0 .. n_inv) inviscid, then the viscous ones,
+  // each in sorted order.
   uint32_t* parts;
   uint32_t* order;
   uint32_t* part;       // per-tile counts of the partition, then its totals

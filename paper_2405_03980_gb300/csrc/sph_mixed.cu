@@ -683,10 +683,10 @@ k_pfilter_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ in
 // collisions at 2.5M particles).  A pass of one neighbour per step took
 // 1.09 ms there (filter and collision model), 8 scalar operations where the
 // packed form issues 4.  The next group of entries is loaded after this
-// one's first pair (before it, 4 % slower: eight more live registers).  Bound
-// by the line lookups of the neighbour gathers (about 37 lines per
-// neighbour of a warp) and by issue: 7.30 -> 7.15 ms at 20.1M with the
-// 256-bit list loads and the decode of entry_vec.
+// one's first pair (before it, 4 % slower: eight more live registers).  It
+// waits on its gathers (L1 72 % and issue 59 % busy, 76 % of the sectors hit):
+// 7.30 -> 7.15 ms at 20.1M with the 256-bit list loads and the decode of
+// entry_vec, 6.98 with the search's candidate order.
 template <int BLOCK, int kOpt>
 __global__ void __launch_bounds__(BLOCK, 512 / BLOCK)
 k_forces_mixed(int64_t n, MixBuf b, MixFields f, const InstDev* __restrict__ inst, NbrWs nw,
