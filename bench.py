@@ -66,8 +66,9 @@ def e2e_steps(workload, steps, override=0):
 # a pair carries (Eqs. 1-2 as the model reads them): two inviscid particles
 # the pressure term alone; unlike species (walls count as viscous) pressure,
 # interfacial and local interaction with its torque; two viscous particles
-# pressure, shear and rotational with its torque.  The FP64 form's pair pass
-# runs one specialised loop per class and these are its counts.  For the
+# pressure, shear and rotational with its torque.  These are the counts of
+# specialised FP64 loops, one per class (the fixed-point pass does the same
+# work in integer instructions).  For the
 # mixed form the same terms cost 6 more (the pair vector from the cell
 # offsets: a subtraction and a fused multiply-add per axis where the FP64
 # form subtracts) plus its compensated sums (4 operations per sum per group
@@ -122,18 +123,21 @@ SEARCH_ALGO_BYTES_PER_PARTICLE = {"fp64": 16, "mixed": 16}
 # only while the kernel's sources hash to the values recorded with it; after
 # any change the roofline reports traffic null until it is re-measured.
 DRAM_BYTES_PER_PARTICLE = {
-    "k_cell_search<true>": (222.4, {"sph_search.cu": "cf8572358b743c10",
-                                    "sph_internal.h": "1756e1381f18b6ad"}),
-    "k_cell_search<false>": (None, {}),
-    "k_density_mixed": (769.9, {"sph_mixed.cu": "701e6e1044459c54",
-                                "sph_internal.h": "1756e1381f18b6ad"}),
-    "k_forces_mixed": (None, {}),
-    "k_forces_mixed_x2": (416.8, {"sph_mixed.cu": "701e6e1044459c54",
-                                  "sph_internal.h": "1756e1381f18b6ad"}),
-    "k_density_fp64": (646.8, {"sph_fp64.cu": "2b1a99c0f5cfa53b",
-                               "sph_internal.h": "1756e1381f18b6ad"}),
-    "k_forces_fp64": (860.5, {"sph_fp64.cu": "2b1a99c0f5cfa53b",
-                              "sph_internal.h": "1756e1381f18b6ad"}),
+    "k_cell_search": (222.6, {"sph_search.cu": "764fce7b782403f0",
+                              "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_cell_search64": (194.9, {"sph_search.cu": "764fce7b782403f0",
+                                "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_density_mixed": (774.4, {"sph_mixed.cu": "5582ad1e7bfa79a9",
+                                "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_forces_mixed": (417.4, {"sph_mixed.cu": "5582ad1e7bfa79a9",
+                               "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_density_fp64": (657.8, {"sph_fp64.cu": "22b15359a02867e1",
+                               "sph_fixed.cuh": "da7c2d15ff1f6f0b",
+                               "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_forces_fx": (952.7, {"sph_fp64.cu": "22b15359a02867e1",
+                            "sph_fixed.cuh": "da7c2d15ff1f6f0b",
+                            "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_forces_fp64": (None, {}),
 }
 
 
@@ -202,14 +206,18 @@ def ratio(traffic, algorithmic):
 # beside the FMA-rate fraction under the same source-hash condition as the
 # traffic.
 BINDING = {
-    "k_forces_mixed_x2": "L1 data path of the neighbour gathers: L1 throughput 81 %, issue "
-                         "58 %, FMA pipe 45 % (ncu, 2,525,900-particle cylinder); each pair is "
-                         "evaluated from both sides",
-    "k_density_mixed": "L1 data path of the offset gathers: L1 throughput 84 %, issue 57 %, "
-                       "FMA pipe 26 % (ncu, 2,525,900-particle cylinder)",
-    "k_forces_fp64": "FP64 pipe 89 % busy (ncu, 2,525,900-particle cylinder); each pair is "
-                     "evaluated from both sides",
-    "k_density_fp64": "FP64 pipe 85 % busy (ncu, 2,525,900-particle cylinder)",
+    "k_forces_mixed": "latency and line lookups of the neighbour gathers: L1 throughput 72 %, "
+                      "issue 60 %, 15 warps per SM (ncu, 2,525,900-particle cylinder); each pair "
+                      "is evaluated from both sides",
+    "k_density_mixed": "latency and line lookups of the offset gathers: L1 throughput 78 %, issue "
+                       "65 %, 27 warps per SM (ncu, 2,525,900-particle cylinder)",
+    "k_forces_fx": "issue of the fixed-point pair geometry and sums on the integer pipe (issue "
+                   "52 %, L1 53 %, FP64 pipe 7 %; ncu, 2,525,900-particle cylinder): the FMA-rate "
+                   "fraction compares the work done and may pass 1; each pair is evaluated from "
+                   "both sides",
+    "k_density_fp64": "issue of the fixed-point geometry on the integer pipe (issue 68 %, FP64 "
+                      "pipe 11 %; ncu, 2,525,900-particle cylinder): the FMA-rate fraction "
+                      "compares the work done and may pass 1",
 }
 
 
