@@ -131,10 +131,10 @@ DRAM_BYTES_PER_PARTICLE = {
                                 "sph_internal.h": "286e6bd5d58bd3e4"}),
     "k_forces_mixed": (417.4, {"sph_mixed.cu": "5582ad1e7bfa79a9",
                                "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_density_fp64": (657.8, {"sph_fp64.cu": "22b15359a02867e1",
+    "k_density_fp64": (657.8, {"sph_fp64.cu": "a5ab8bffef1ad845",
                                "sph_fixed.cuh": "da7c2d15ff1f6f0b",
                                "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_forces_fx": (952.7, {"sph_fp64.cu": "22b15359a02867e1",
+    "k_forces_fx": (952.7, {"sph_fp64.cu": "a5ab8bffef1ad845",
                             "sph_fixed.cuh": "da7c2d15ff1f6f0b",
                             "sph_internal.h": "286e6bd5d58bd3e4"}),
     "k_forces_fp64": (None, {}),

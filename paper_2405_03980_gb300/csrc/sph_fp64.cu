@@ -365,7 +365,7 @@ __device__ __noinline__ void density_exact(int64_t n, int64_t i, uint32_t t0, ui
 // FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18 of its value
 // (an FP64 evaluation within a few 1.1e-16), and the sum over a list is
 // exact.  20.1M particles: 64.5 ms with FP64 arithmetic, 19.6 ms in fixed
-// point with a thread per particle, 14.5 ms now (bound by issue, 68 %, and the
+// point with a thread per particle, 14.0 ms now (bound by issue, 68 %, and the
 // ALU).  Lists written by the search instead took 10.5 ms here but 7.2 ms more
 // there.  kFilter: some instance uses the pressure filter; the kernel shape of
 // every list entry is then stored beside the list (nw.wsh_d).
@@ -848,7 +848,7 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // particles, 0 to 300 steps): relative L2 error of the acceleration 8e-16 to
 // 6e-15 (FP64 loops 3e-15 to 3e-14), of the spin change 2.0e-16 to 2.4e-16
 // (4.1e-16 to 8.1e-16), of the density 7e-17 (3.6e-16).  20.1M particles:
-// 134.3 ms before, 38.6 ms now.
+// 134.3 ms before, 37.4 ms now.
 
 // Particles below which eight and four lanes take a list, else two: more lanes
 // fill the GPU sooner, fewer spend less on adding up (pair pass with 8 / 4 / 2
