@@ -425,8 +425,10 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
   uint32_t parts = part0 | ((part1 - part0) << 11);
   bool in_memory = cnt > kStaged;  // the list, past the staging
   __syncwarp();
-  if (in_memory) {  // rounds before the staging filled up wrote to it alone
-    for (uint32_t t = (uint32_t)lane; t < kStaged && t < (uint32_t)nw.cap; t += kLanes)
+  // rounds before the staging filled up wrote to it alone (a list past the
+  // capacity is written anew below, by one lane)
+  if (in_memory && cnt <= (uint32_t)nw.cap) {
+    for (uint32_t t = (uint32_t)lane; t < kStaged; t += kLanes)
       nw.list[nbr_slot(n, i, t)] = staged[row][t];
   }
   if (cnt > (uint32_t)nw.cap) {
