@@ -4,15 +4,20 @@
 // integer and FP32 rate, so the FP64 form's loops over neighbours were bound
 // by the FP64 pipe (85-89 % busy).  The geometry of a pair is bounded by the
 // kernel support (r < 2h), so it needs no exponent: lengths are held in units
-// of 2h as signed 64-bit integers with 62 fractional bits, nine more than a
-// double's mantissa has, and the distance, the kernel shapes and the sums are
-// formed on the integer pipe, each product rounded at 2^-60 or finer.
+// of 2h as signed 64-bit integers with 62 fractional bits, nine more than the
+// mantissa of a double between 1/2 and 1 has, and the distance, the kernel
+// shapes and the sums are formed on the integer pipe.
 //
 //  - A coordinate x is x / (2h) 2^62 modulo 2^64.  Differences of
 //    coordinates are exact modulo 2^64, which holds every difference below
 //    2 (2h); so the range of the box costs no precision.
 //  - r^2 is in units of 2^-60 (2h)^2, r in units of 2^-62 2h.
 //  - The kernel shapes with t = 1 - r / 2h: F shape t^3, W shape t^4 (5 - 4t).
+//    Near the cutoff they are far below one, where an absolute step is coarse:
+//    the density and the filter, which the self term keeps away from zero, take
+//    W at steps of 2^-61, the pair pass scales t up first (scaled_t).  What is
+//    left there is the error of t itself, 2^-58.6 / t of its value (that of an
+//    FP64 evaluation is about 2^-53 / t).
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -172,6 +177,20 @@ SPH_FX u64 shape_w8(u64 t, u64 t2) {
   return mulhi(mulhi(t2, t2), 0xA000000000000000ull - (t >> 1));
 }
 
+// Shapes scaled up by a power of two, which keep their precision where t is
+// small: with T = t 2^lead, the F shape is mulhi(mulhi(T, T), T) 2^(-3 lead)
+// and the W shape over 8 is shape_w8(t, mulhi(T, T)) 2^(-4 lead).
+SPH_FX u64 scaled_t(u64 t, uint32_t lead) { return t << lead; }
+// Leading zeros of a 64-bit value, 32 at most: of t, the lead that brings it
+// into [1/2, 1), or up by 2^32.
+SPH_FX uint32_t lead32(u64 v) {
+#ifdef __CUDA_ARCH__
+  return (uint32_t)__clz((int)(uint32_t)(v >> 32));
+#else
+  return (v >> 32) ? (uint32_t)__builtin_clz((uint32_t)(v >> 32)) : 32u;
+#endif
+}
+
 // Sum of W shapes (over 8, 2^-64) in 96 bits, and its value.
 struct Sum96 {
   uint32_t w0 = 0, w1 = 0, w2 = 0;
@@ -263,16 +282,6 @@ SPH_FX i64 mantissa_at(double x, int e) {
   const int s = e - (ex - 1022);
   const u64 q = s < 63 ? m >> s : 0ull;
   return (i64)((b >> 63) ? 0ull - q : q);
-}
-
-// Leading zeros of a positive value below 2^62, counted from bit 61, 24 at most.
-SPH_FX int lead62(u64 v) {
-#ifdef __CUDA_ARCH__
-  const int z = __clz((int)(uint32_t)(v >> 32)) - 2;
-#else
-  const int z = ((v >> 32) ? __builtin_clz((uint32_t)(v >> 32)) : 32) - 2;
-#endif
-  return z < 24 ? z : 24;
 }
 
 // Signed sum in 96 bits.

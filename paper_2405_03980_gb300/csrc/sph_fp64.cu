@@ -445,8 +445,10 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
   __syncwarp();
   if (live && lane == 0) nw.count[i] = cnt;
   // ---- the sum
-  const uint32_t na = part_inv(parts);
+  const uint32_t na = part_inv(parts), nab = na + part_vis(parts);
   fx::Sum96 sum[2];  // the inviscid neighbours, the others
+  uint32_t bits[3] = {0u, 0u, 0u};  // high halves of the t of each class, joined: the highest bit
+                                    // is the largest t's
   uint32_t dead = 0;
   bool undecided = false;
   const auto entry = [&](uint32_t t) {
@@ -468,8 +470,15 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
       if (r2 - R.near2 < R.width) {
         const uint64_t tt = fx::shape_t(r2);
         w8 = fx::shape_w8(tt, fx::mulhi(tt, tt));
-        if (t < na) sum[0].add(w8);
-        else sum[1].add(w8);
+        const uint32_t hi = (uint32_t)(tt >> 32);
+        if (t < na) {
+          sum[0].add(w8);
+          bits[0] |= hi;
+        } else {
+          sum[1].add(w8);
+          bits[1] |= t < nab ? hi : 0u;
+          bits[2] |= t < nab ? 0u : hi;
+        }
       } else if (r2 >= R.far2) {
         ent = (uint32_t)i | (21u << kNbrIndexBits);
         ++dead;
@@ -484,8 +493,11 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
       density_exact<kFilter>(n, i, (uint32_t)lane, na, cnt, b.pos, &P, &nw, &R, sum, &dead);
   }
   __syncwarp();
+  uint32_t lead = (uint32_t)(__clz((int)bits[0]) | (__clz((int)bits[1]) << 8) |
+                             (__clz((int)bits[2]) << 16));
 #pragma unroll
   for (int o = 1; o < kLanes; o <<= 1) {
+    lead = __vminu4(lead, __shfl_xor_sync(~0u, lead, o));
     dead += __shfl_xor_sync(~0u, dead, o);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -496,6 +508,7 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
     }
   }
   if (lane < 2) sums[row][lane] = lane == 0 ? sum[0].shape_sum() : sum[1].shape_sum();
+  if (live && lane == 0) nw.lead[i] = lead;
   if (lane == 0) gone[row] = parts | (min(dead, 1023u) << 22);
   __syncthreads();
   // ---- rho and P, one thread per particle
@@ -830,11 +843,16 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // exponent; a first walk over i's list takes the largest exponents of its
 // neighbours, and the largest |v_ij| in FP32, which give the power of two
 // 2^E2 above every |u_ij|.  u_ij is then rounded at 2^-60 of that (an FP64
-// evaluation rounds each operation at 2^-53 of its own value), the
-// coefficient V_j F or V_j W that multiplies it is shifted up to 62 bits and
-// the product added that much lower in a 96-bit sum, and a pressure term is
-// rounded at 2^-57 of the largest pressure.  A sum is exact: it does not
-// depend on the order of the list or on the number of lanes.
+// evaluation rounds each operation at 2^-53 of its own value).  The shapes t^3
+// and t^4 (5 - 4t) are formed from t 2^lead, which the largest t of the
+// neighbours' class brings into [1/2, 1) (found by the density pass), so they
+// keep their 60 bits where all neighbours of a class stand near the cutoff
+// and t is small (from t itself the force of one neighbour at t = 0.001 was off
+// by 1.6e-8, its torque by 1.9e-7).  The coefficient V_j F or V_j W of u_ij is
+// shifted up to 62 bits and the product added that much lower in a 96-bit
+// sum; a pressure term is rounded at 2^-58 of the largest pressure and F.  A
+// sum is exact: it does not depend on the order of the list or on the number
+// of lanes.
 //
 // kL lanes take a particle's entries in turn, two to eight of them (warps of 16
 // or 8 particles diverge less than warps of 32, and small vessels spread over
@@ -859,9 +877,7 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 constexpr int64_t kPairLanes8 = 1 << 15;
 constexpr int64_t kPairLanes4 = 1 << 18;
 constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip
-// Entries that a 64-bit sum holds: a pressure term is below 2 (27/256) 2^57 (t^3 (1 - t) is at
-// most 27/256), an interfacial one below (27/256) 2^58.
-constexpr uint32_t kMaxFx = 160;
+constexpr uint32_t kMaxFx = 160;  // longer lists take the FP64 route
 constexpr int kSlots = 48;           // per particle: 3 phases x 12 sums, 12 of the FP64 route
 
 __global__ void k_pair_records(int64_t n, Fp64Buf b, const InstDev* __restrict__ inst, NbrWs nw) {
@@ -975,16 +991,16 @@ __device__ __noinline__ void slow_walk(int64_t n, int64_t i, uint32_t cnt, uint3
   }
 }
 
-// Entries t0, t0 + kL, ... of particle i below t1.
+// Entries t0, t0 + kL, ... of particle i below t1, all of one class; lead:
+// the leading zeros of the class's largest t, from which its scale follows.
 template <int kPath, int kL>
 __device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t n, int64_t i,
-                                        uint32_t t0, uint32_t t1, uint32_t* err,
+                                        uint32_t t0, uint32_t t1, uint32_t lead,
+                                        uint32_t* err,
                                         fx::Acc96 (&acc)[12], bool& any_slow) {
   using fx::Half;
   using fx::mul;
   using fx::split;
-  // the pressure's and the interfacial sums fit 64 bits (kMaxFx terms)
-  int64_t sp[3] = {0, 0, 0}, sx[3] = {0, 0, 0};
   // the next entry's position record is loaded one entry ahead, the entry
   // after it two ahead
   if (t0 >= t1) return;
@@ -1008,13 +1024,14 @@ __device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t
     }
     const int64_t rho = fx::root(r2);
     const uint64_t tt = (uint64_t)((1ll << 62) - rho) << 2;  // t in units of 2^-64
-    const uint64_t tq = fx::mulhi(tt, tt);
-    const uint64_t F64 = fx::mulhi(tq, tt);                  // F shape t^3, 2^-64
+    const uint64_t T = fx::scaled_t(tt, lead);
+    const uint64_t Tq = fx::mulhi(T, T);
+    const uint64_t F = fx::mulhi(Tq, T);                     // F shape t^3 2^(3 lead)
     // pressure: (P_i / rho_i^2 + P_j / rho_j^2) F r_ij
     const int64_t g = C.P + shr(rec->P, C.EP - (int)(q.exps >> 16));
-    const Half gF = split(mul(split(g), split((int64_t)(F64 >> 2))));
+    const Half gF = split(mul(split(g), split((int64_t)(F >> 2))) << 2);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) sp[a] += mul(gF, d[a]);
+    for (int a = 0; a < 3; ++a) acc[a].add(mul(gF, d[a]));
     if (kPath == kPathII) continue;
     // u_ij = v_ij + r_ij x (w_i + w_j) / 2
     const int sv = C.Ev - (int)(q.tag >> 16), sh = C.Eh - (int)(q.exps & 0xFFFFu);
@@ -1029,19 +1046,19 @@ __device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t
     u[1] = split(v[1] + fx::mul_sub(d[2], s[0], d[0], s[2]));
     u[2] = split(v[2] + fx::mul_sub(d[0], s[1], d[1], s[0]));
     const uint64_t V = rec->V << 2;
-    const uint64_t VF = fx::mulhi(V, F64) >> 2;  // V_j F, 2^-62
-    uint64_t c;  // the coefficient of u: V_j W (unlike species) or V_j F (two viscous)
+    const uint64_t VF = fx::mulhi(V, F);
+    uint64_t c;  // the coefficient of u: V_j W / 8 (unlike species) or V_j F (two viscous), 2^-64
     if (kPath == kPathIX) {
       // interfacial: V_j F r_ij
       const Half VFh = split((int64_t)(VF >> 2));
 #pragma unroll
-      for (int a = 0; a < 3; ++a) sx[a] += mul(VFh, d[a]);
-      c = fx::mulhi(V, fx::shape_w8(tt, tq)) << 1;
+      for (int a = 0; a < 3; ++a) acc[3 + a].add(mul(VFh, d[a]));
+      c = fx::mulhi(V, fx::shape_w8(tt, Tq));
     } else {
       c = VF;
     }
-    const int lz = fx::lead62(c), up = 24 - lz;  // 2^lz c has 62 bits
-    const Half ch = split((int64_t)(c << lz));
+    const int lz = (int)min(fx::lead32(c), 24u), up = 24 - lz;
+    const Half ch = split((int64_t)((c << lz) >> 2));  // 2^lz c in 62 bits
     if (kPath == kPathVV) {
       // the part along e_ij: V_j F (e_ij . v_ij) e_ij
       const Half z = split(fx::recip(rho));
@@ -1066,11 +1083,6 @@ __device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t
     acc[9].add_shifted(fx::mul_sub(d[1], ph[2], d[2], ph[1]), up);
     acc[10].add_shifted(fx::mul_sub(d[2], ph[0], d[0], ph[2]), up);
     acc[11].add_shifted(fx::mul_sub(d[0], ph[1], d[1], ph[0]), up);
-  }
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    acc[a].add(sp[a]);
-    if (kPath == kPathIX) acc[3 + a].add(sx[a]);
   }
 }
 
@@ -1118,7 +1130,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const bool inv_i = first + row < n_inv;
   const int64_t i = live ? checked_index(nw.order[first + row], n, err) : 0;
   const InstDev& P = inst[b.inst[i]];
-  uint32_t cnt = 0, na = 0, nb = 0;
+  uint32_t cnt = 0, na = 0, nb = 0, leads = 0;
   FxCtx C;
   C.q = ld_qpos(nw.posq + i);
   if (live) {
@@ -1126,6 +1138,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     const uint32_t parts = nw.parts[i];
     na = min(part_inv(parts), cnt);
     nb = min(part_vis(parts), cnt - na);
+    leads = nw.lead[i];
   }
   // first walk: the largest exponents, and the largest |v_ij|
   const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
@@ -1202,6 +1215,8 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     fx::Acc96 acc[12];
     const uint32_t t0 = ph == 0 ? end[0] : (ph == 1 ? end[1] : end[2]);
     const uint32_t t1 = ph == 0 ? end[1] : (ph == 1 ? end[2] : end[3]);
+    const uint32_t lead = (leads >> (8 * ph)) & 0xFFu;
+    const int s3 = 3 * (int)lead, s4 = 4 * (int)lead;  // the scales of F and W
     if (!__any_sync(~0u, t0 < t1)) {  // none for this warp's particles
 #pragma unroll
       for (int k = 0; k < kKeep; ++k) sums[row][12 * ph + kKeep * part + k] = 0.0;
@@ -1209,14 +1224,14 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     }
     if (inv_i) {
       if (ph == 0)
-        fx_loop<kPathII, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
+        fx_loop<kPathII, kL>(C, nw, n, i, t0 + lane, t1, lead, err, acc, any_slow);
       else
-        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
+        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, lead, err, acc, any_slow);
     } else {
       if (ph == 0)
-        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
+        fx_loop<kPathIX, kL>(C, nw, n, i, t0 + lane, t1, lead, err, acc, any_slow);
       else
-        fx_loop<kPathVV, kL>(C, nw, n, i, t0 + lane, t1, err, acc, any_slow);
+        fx_loop<kPathVV, kL>(C, nw, n, i, t0 + lane, t1, lead, err, acc, any_slow);
     }
     __syncwarp();
     if (ph == 0 && __all_sync(~0u, inv_i)) {  // pairs of inviscid particles: pressure alone
@@ -1231,18 +1246,19 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
 #pragma unroll
         for (int q = 1; q < kL && k + q < 3; ++q)
           if (lane == q) mine = acc[k + q];
-        if (k + lane < 3) sums[row][k + lane] = mine.value(E_P - 57);
+        if (k + lane < 3) sums[row][k + lane] = mine.value(E_P - 59 - s3);
       }
       continue;
     }
     reduce12<kL>(acc);
-    // the pressure's sums are in units of 2^(E_P - 57), the interfacial
-    // force's of 2^-58, the torque's of 2^(E2 - 84), the others' of 2^(E2 - 83)
+    // the units of the sums: the pressure's, the interfacial force's (unlike
+    // species) or the part along e_ij's, that along u_ij's, the torque's
     const bool unlike = inv_i ? ph > 0 : ph == 0;
+    const int eu = unlike ? E2 - 80 - s4 : E2 - 83 - s3;
 #pragma unroll
     for (int k = 0; k < kKeep; ++k) {
       const int q = kKeep * part + k;
-      const int e = q < 3 ? E_P - 57 : (q < 6 ? (unlike ? -58 : E2 - 83) : (q < 9 ? E2 - 83 : E2 - 84));
+      const int e = q < 3 ? E_P - 59 - s3 : (q < 6 ? (unlike ? -60 - s3 : eu) : (q < 9 ? eu : eu - 1));
       sums[row][12 * ph + q] = acc[k].value(e);
     }
   }

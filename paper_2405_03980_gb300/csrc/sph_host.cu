@@ -401,6 +401,7 @@ void carve(void* state, void* ws, int32_t n_inst, int64_t n, int64_t n_cells,
     c.f.vp = w.take<dvec2>(n);
     // the split lists and the species order of the FP64 pair pass
     c.nw.parts = w.take<uint32_t>(n);
+    c.nw.lead = w.take<uint32_t>(n);
     c.nw.order = w.take<uint32_t>(n);
     c.nw.part = w.take<uint32_t>(2 * ((n + kPartTile - 1) / kPartTile) + 2);
   } else {

@@ -247,6 +247,8 @@ struct NbrWs {
   // for the pair pass: order[0 .. n_inv) inviscid, then the viscous ones,
   // each in sorted order.
   uint32_t* parts;
+  uint32_t* lead;       // leading zeros of the largest t = 1 - r / 2h of each class, 8 bits
+                        // each, 32 at most, for the pair pass's scales
   uint32_t* order;
   uint32_t* part;       // per-tile counts of the partition, then its totals
   float4* posf;         // FP32 copy of sorted positions (FP64-form prefilter)

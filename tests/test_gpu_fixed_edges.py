@@ -49,3 +49,97 @@ def test_prefiltered_lists_past_the_capacity(m, cap):
     print(per_particle_check(sim.state_arrays(), c, 0))
     assert neighbours_equal(sim, c)
     sim.close()
+
+
+def exact_sites(c, m):
+    """Acceleration and spin change of every particle, and the sums of the
+    magnitudes of their pair terms, for consecutive groups of m particles that
+    see nothing but each other, in extended precision."""
+    L = np.longdouble
+    q, p = c.params, oracle.make_params(c.params)
+    n = len(c.species)
+    h, aD = L(q["h"]), L(oracle.W(p, 0.0))
+    mass = np.where(c.species == 0, oracle.mass(p, 0), oracle.mass(p, 1)).astype(L).reshape(-1, m)
+    inv = (c.species == 0).reshape(-1, m)
+    x, v, w = (a.astype(L).reshape(-1, m, 3) for a in (c.pos, c.vel, c.spin))
+    d = x[:, :, None] - x[:, None]
+    r = np.sqrt((d * d).sum(-1))
+    t = 1 - r / (2 * h)
+    t[t < 0] = 0
+    self_ = np.eye(m, dtype=bool)[None]
+    W = aD * t**4 * (5 - 4 * t)
+    rho = (W * mass[:, None]).sum(-1)
+    P = L(q["p0"]) * (rho / L(q["rho0"])) ** int(q["alpha_P"]) - L(q["beta_P"])
+    V, Pr = mass / rho, P / rho**2
+    F = 5 * aD / h**2 * t**3 * ~self_
+    W = W * ~self_
+    VV = V[:, :, None] * V[:, None]
+    u = v[:, :, None] - v[:, None]
+    dv = (d * u).sum(-1)
+    s = (w[:, :, None] + w[:, None]) / 2
+    u = u + np.cross(d, s)
+    unlike = inv[:, :, None] != inv[:, None]
+    vv = ~inv[:, :, None] & ~inv[:, None]
+    A, Bv = 10 * (L(q["eta_bar"]) - L(0.6) * L(q["eta_r"])), 4 * L(q["eta_r"])
+    r2 = np.where(self_, 1, r * r)
+    along = (mass[:, :, None] * mass[:, None] * (Pr[:, :, None] + Pr[:, None]) * F
+             + vv * (Bv - A) * VV * F * dv / r2)
+    bu = np.where(unlike, -L(q["C_l"]) * VV * W, -(vv * Bv * VV * F))
+    aT = unlike * L(q["C_T"]) * VV * F
+    rot = bu[..., None] * u
+    f = along[..., None] * d + rot + aT[..., None] * d * np.array([1, 1, 0])
+    tau = -np.cross(d, rot) / 2
+    I = L(q["inertia_coef"]) * mass * L(q["dx"]) ** 2
+    out = []
+    for g, k in ((f, mass), (tau, I)):
+        out += [(g.sum(2) / k[..., None]).reshape(n, 3), (np.linalg.norm(g.astype(float), axis=-1).sum(2) / k.astype(float)).reshape(n)]
+    return out
+
+
+def sites(kind, t, seed):
+    """Groups of particles 9 apart.  "pairs": two particles of any species at
+    r = 2h (1 - t).  "one unlike": an inviscid particle among seven others and
+    one viscous particle at that distance, on which alone its torque hangs."""
+    rng = np.random.default_rng(seed)
+    S = len(t)
+    e = rng.normal(size=(S, 8, 3))
+    e /= np.linalg.norm(e, axis=-1, keepdims=True)
+    far = 2.6 * (1 - t)[:, None] * e[:, 0]
+    if kind == "pairs":
+        off, sp = np.stack([np.zeros((S, 3)), far], 1), rng.integers(0, 2, (S, 2))
+    else:
+        off = np.concatenate([np.zeros((S, 1, 3)), rng.uniform(0.9, 1.6, (S, 7, 1)) * e[:, 1:],
+                              far[:, None]], 1)
+        sp = np.zeros((S, 9), dtype=int)
+        sp[:, 8] = 1
+    k = int(np.ceil(np.sqrt(S)))
+    at = np.stack([np.arange(S) % k - k / 2, np.arange(S) // k - k / 2, np.zeros(S)], 1) * 9.0
+    off = off + at[:, None] + [0.0, 0.0, 4.0]
+    return off.reshape(-1, 3), sp.ravel(), off.shape[1], (9.0 * k / 2 + 9.0,) * 2
+
+
+@pytest.mark.parametrize("kind", ["pairs", "one unlike"])
+def test_sums_that_hang_on_pairs_near_the_cutoff(kind):
+    """Force and torque relative to their own pair terms, whatever t.  The
+    fixed-point r is within 2^-58.6 of 2h (positions to a unit of 2^-62 each,
+    r^2 to three of 2^-60), which t^4 turns into 2^-56.6 / t; the coefficients
+    (density, Tait power, volumes) are FP64 operations, some forty of 2^-53."""
+    t = 10.0 ** np.random.default_rng(2).uniform(-6.0, -0.3, 900)
+    pos, sp, m, half = sites(kind, t, 4)
+    c = box_of(pos, sp, half)
+    sim = sim_of(c)
+    st = sim.state_arrays()
+    acc, sa, dsp, sd = exact_sites(c, m)
+    for f, ref, s in (("acc", acc, sa), ("dspin", dsp, sd)):
+        e = np.linalg.norm((st[f] - ref).astype(float), axis=1)
+        assert np.array_equal(e[s == 0], np.zeros((s == 0).sum()))
+        tt = np.repeat(t, m)
+        rows = s > 0
+        if kind == "one unlike":
+            rows &= np.arange(len(s)) % m == 0   # the particle in the middle
+            tt = tt if f == "dspin" else np.full(len(s), 0.3)
+        bound = 5e-15 + 2.0**-56 / tt
+        worst = (e[rows] / s[rows] / bound[rows]).max()
+        print(kind, f, "largest error over its bound", worst)
+        assert rows.sum() > 200 and worst <= 1.0
+    sim.close()
