@@ -984,6 +984,7 @@ __device__ __noinline__ void slow_walk(int64_t n, int64_t i, uint32_t cnt, uint3
                                        const FxCtx* C, double* out) {
   for (uint32_t t = 0; t < cnt; ++t) {
     const uint32_t ent = nw->list[nbr_slot(n, i, t)], j = ent & kNbrIndexMask;
+    if ((int64_t)j == i) continue;  // beyond 2h
     const PairVec v = pair_vec(C->q, nw->posq[j], ent, C->R);
     const uint64_t r2 = fx::norm2(v.d[0], v.d[1], v.d[2]);
     if (t >= vv ? r2 - kNearVV < C->width_vv : r2 - C->R.near2 < C->R.width) continue;
@@ -1019,7 +1020,7 @@ __device__ __forceinline__ void fx_loop(const FxCtx& C, const NbrWs& nw, int64_t
     const Half(&d)[3] = pv.d;
     const uint64_t r2 = fx::norm2(d[0], d[1], d[2]);
     if (kPath == kPathVV ? r2 - kNearVV >= C.width_vv : r2 - C.R.near2 >= C.R.width) {
-      any_slow = true;
+      any_slow |= (int64_t)j != i;  // (an entry beyond 2h names i, and adds nothing)
       continue;
     }
     const int64_t rho = fx::root(r2);
