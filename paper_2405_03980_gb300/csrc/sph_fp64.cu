@@ -877,7 +877,6 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 constexpr int64_t kPairLanes8 = 1 << 15;
 constexpr int64_t kPairLanes4 = 1 << 18;
 constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip
-constexpr uint32_t kMaxFx = 160;  // longer lists take the FP64 route
 constexpr int kSlots = 48;           // per particle: 3 phases x 12 sums, 12 of the FP64 route
 
 __global__ void k_pair_records(int64_t n, Fp64Buf b, const InstDev* __restrict__ inst, NbrWs nw) {
@@ -1188,9 +1187,8 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const bool still = (ev | eh) == 0u;
   const int E2 = still ? -1020 : max((int)(__float_as_uint(bound) >> 23) - 126, E_h + 2);
   const int E_v1 = max(E_v, E2);
-  // values the scales do not cover (a longer list than the sums hold,
-  // overflow, NaN, FP32 underflow of v_ij)
-  const bool covered = cnt <= kMaxFx && eP < 2047u && ev < 2047u && eh < 2047u &&
+  // values the scales do not cover (overflow, NaN, FP32 underflow of v_ij)
+  const bool covered = eP < 2047u && ev < 2047u && eh < 2047u &&
                        bound < 1e30f && (still || bound > 1e-30f);
   {
     C.R = pair_range(P, z_cell(P, cw.skey[i]));

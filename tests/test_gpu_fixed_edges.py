@@ -143,3 +143,15 @@ def test_sums_that_hang_on_pairs_near_the_cutoff(kind):
         print(kind, f, "largest error over its bound", worst)
         assert rows.sum() > 200 and worst <= 1.0
     sim.close()
+
+
+def test_lists_of_a_thousand_neighbours():
+    """The sums hold every list that the capacity admits."""
+    rng = np.random.default_rng(11)
+    e = rng.normal(size=(1000, 3))
+    pos = 1.25 * e / np.linalg.norm(e, axis=1)[:, None] * rng.uniform(0, 1, (1000, 1)) ** (1 / 3)
+    c = box_of(pos + [0.0, 0.0, 4.0], rng.integers(0, 2, 1000), (8.0, 8.0))
+    sim = sim_of(c, nbr_cap=1024)
+    print(per_particle_check(sim.state_arrays(), c, 0))
+    assert neighbours_equal(sim, c)
+    sim.close()
