@@ -351,6 +351,34 @@ __device__ __noinline__ void density_exact(int64_t n, int64_t i, uint32_t t0, ui
   }
 }
 
+// The density of a particle that weighs little against a neighbour's own term
+// (species masses far apart): its sum hangs on W shapes far below one, where
+// the fixed-point step of 2^-61 shows.  Its list once more in FP64, with the
+// filter's shapes.
+template <bool kFilter>
+__device__ __noinline__ double density_light(int64_t n, int64_t i, uint32_t na, uint32_t skey,
+                                             const dvec4* pos, const InstDev* Pp,
+                                             const NbrWs* nwp, double m_i) {
+  const InstDev& P = *Pp;
+  const NbrWs& nw = *nwp;
+  const PairRange R = pair_range(P, z_cell(P, skey));
+  const dvec4 a = pos[i];
+  const uint32_t cnt = nw.count[i];
+  double S[2] = {0.0, 0.0};
+  for (uint32_t t = 0; t < cnt; ++t) {
+    const int64_t at = nbr_slot(n, i, t);
+    const uint32_t ent = nw.list[at], j = ent & kNbrIndexMask;
+    if ((int64_t)j == i) continue;
+    const bool across = (ent >> (kNbrIndexBits + 4)) == R.wrap_code;
+    const double r = sqrt(exact_r2(a, pos[j], across, R, P));
+    const double t1 = fma(-0.5 * P.inv_h, r, 1.0), t2 = t1 * t1;
+    const double W = t2 * t2 * fma(2.0 * P.inv_h, r, 1.0);
+    S[t < na ? 0 : 1] += W;
+    if (kFilter) nw.wsh_d[at] = W;
+  }
+  return fma(P.m_s * P.aD, S[0], fma(P.m_n * P.aD, S[1], m_i * P.aD));
+}
+
 // Density and Tait pressure (Eq. 4).  kLanes lanes first turn the particle's
 // candidate mask (the search's FP32 prefilter; words dealt out to the lanes)
 // into its list, inviscid neighbours, then viscous ones, then walls, in shared
@@ -508,7 +536,7 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
     }
   }
   if (lane < 2) sums[row][lane] = lane == 0 ? sum[0].shape_sum() : sum[1].shape_sum();
-  if (live && lane == 0) nw.lead[i] = lead;
+  if (live && lane == 0) nw.lead[i] = lead | (P.fx_pairs ? 0u : 1u << 31);
   if (lane == 0) gone[row] = parts | (min(dead, 1023u) << 22);
   __syncthreads();
   // ---- rho and P, one thread per particle
@@ -523,6 +551,9 @@ k_density_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
   if (sp != 3)
     rho = fma(Q.m_s * Q.aD, sums[threadIdx.x][0],
               fma(Q.m_n * Q.aD, sums[threadIdx.x][1], m_i * Q.aD));
+  if (rho < Q.rho_light && sp != 3)
+    rho = density_light<kFilter>(n, io, part_inv(gone[threadIdx.x]), cw.skey[io], b.pos, &Q, &nw,
+                                 m_i);
   nw.parts[io] = gone[threadIdx.x];
   const double Pres = Q.p0 * ipow(rho * Q.inv_rho0, Q.alphaP) - Q.beta_P;
   f.rho[io] = rho;
@@ -765,6 +796,7 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
   C.pi = b.pos[i];
   const int sp_i = (int)C.pi.w;
   const InstDev& P = inst[b.inst[i]];
+  if (P.fx_pairs) return;  // by k_forces_fx
   C.vi = b.vel[i];   // w = V_i
   C.wi = b.spin[i];  // w = P_i / rho_i^2
   const double m_i = sp_i == 0 ? P.m_s : P.m_n;
@@ -1139,6 +1171,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     na = min(part_inv(parts), cnt);
     nb = min(part_vis(parts), cnt - na);
     leads = nw.lead[i];
+    if (leads >> 31) cnt = na = nb = 0;  // an instance of k_forces_fp64's
   }
   // first walk: the largest exponents, and the largest |v_ij|
   const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
@@ -1281,6 +1314,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const int64_t io = checked_index(nw.order[first + threadIdx.x], n, err);
   const bool inv_o = first + threadIdx.x < n_inv;
   const InstDev& Q = inst[b.inst[io]];
+  if (!Q.fx_pairs) return;
   const uint32_t fl = Q.flags;
   const double m_i = inv_o ? Q.m_s : Q.m_n, V_i = b.vel[io].w, two_h = 2.0 * Q.h;
   const double mc = (fl & SPH_TERM_P) ? m_i * Q.cF * two_h : 0.0;
@@ -1435,9 +1469,9 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
   if (e != cudaSuccess) return e;
   const unsigned g256 = (unsigned)((n + 255) / 256), g128 = (unsigned)((n + 127) / 128),
                  g64 = (unsigned)((n + 63) / 64);
-  // the pair pass carries only the options some instance uses
-  const int opt = (lc.any_literal ? kOptLiteral : 0) | (lc.any_collision ? kOptCollision : 0);
-  if (opt == 0) {  // the default form, in fixed point
+  // each instance's pairs by one of the two passes, by its own parameters (so
+  // that a batched instance's bits equal its solo run's)
+  if (lc.any_fixed) {
     k_pair_records<<<grid_for(n, 256, lc.sm_count, 32), 256, 0, s>>>(n, b, inst, nw);
     auto fixed = [&](auto lanes) {
       constexpr int L = decltype(lanes)::value;
@@ -1456,22 +1490,27 @@ cudaError_t launch_forces_fp64(int64_t n, const Fp64Buf& b, const Fp64Fields& f,
     else
       fixed(std::integral_constant<int, 2>());
     if (launches) *launches += 2;
-    return cudaGetLastError();
   }
-  auto go = [&](auto kopt) {
-    constexpr int O = decltype(kopt)::value;
-    if (lc.block_forces == 256)
-      k_forces_fp64<256, O><<<g256, 256, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
-    else if (lc.block_forces == 64)
-      k_forces_fp64<64, O><<<g64, 64, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
-    else
-      k_forces_fp64<128, O><<<g128, 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
-  };
-  if (opt == kOptCollision)
-    go(std::integral_constant<int, kOptCollision>());
-  else  // the literal F_sn, with or without collisions
-    go(std::integral_constant<int, kOptLiteral | kOptCollision>());
-  if (launches) ++*launches;
+  if (lc.any_loops) {
+    auto go = [&](auto kopt) {
+      constexpr int O = decltype(kopt)::value;
+      if (lc.block_forces == 256)
+        k_forces_fp64<256, O><<<g256, 256, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+      else if (lc.block_forces == 64)
+        k_forces_fp64<64, O><<<g64, 64, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+      else
+        k_forces_fp64<128, O><<<g128, 128, 0, s>>>(n, b, f, inst, cw, nw, err, 2 * nt);
+    };
+    // the loops carry only the options some instance uses
+    const int opt = (lc.any_literal ? kOptLiteral : 0) | (lc.any_collision ? kOptCollision : 0);
+    if (opt == 0)
+      go(std::integral_constant<int, 0>());
+    else if (opt == kOptCollision)
+      go(std::integral_constant<int, kOptCollision>());
+    else  // the literal F_sn, with or without collisions
+      go(std::integral_constant<int, kOptLiteral | kOptCollision>());
+    if (launches) ++*launches;
+  }
   return cudaGetLastError();
 }
 

@@ -201,7 +201,20 @@ sph_status derive(const sph_params& p, InstDev& d) {
     d.fx_near = fx::kNear2;
     d.fx_width = ok ? fx::kOne2 - band - fx::kNear2 : 0u;
     d.fx_far = ok ? fx::kOne2 + band : ~0ull;
+    // The pair pass brings a list's volumes and pressures to common scales,
+    // with the bits to spare for a few powers of two between them: species
+    // whose masses are further apart than eight, whose P / rho^2 can differ by
+    // the square of that in one list, keep the FP64 loops (at a ratio of 1000
+    // an acceleration in fixed point was off by up to 1.5e-14 of its pair terms,
+    // FP64 by 1.3e-15).  So do the options that fixed point does not carry, and
+    // boxes where it decides no pair.
+    d.fx_pairs = ok && p.mass_ratio >= 0.125 && p.mass_ratio <= 8.0 &&
+                 !(p.flags & (SPH_SN_LITERAL | SPH_COLLISION));
   }
+
+  // 2^-8 of the heavier species' own term (no density is lower at like masses)
+  d.rho_light = ldexp(d.aD * fmax(d.m_s, d.m_n), -8);
+  if (d.aD * fmin(d.m_s, d.m_n) >= d.rho_light) d.rho_light = 0.0;
 
   // FP32 constants of the mixed form
   if (p.precision == SPH_MIXED &&
@@ -871,11 +884,14 @@ sph_status sph_init_batch(sph_ctx** out, int32_t n_inst, const sph_params* param
   c->lc.block_forces = 128;
   c->lc.search_warps = 4;
   c->lc.search_depth = 512;
+  c->lc.any_fixed = false;
+  c->lc.any_loops = false;
   c->lc.any_literal = false;
   c->lc.any_collision = false;
   c->lc.any_filter = false;
   for (const InstDev& d : pl.inst) {
     c->max_cells = std::max(c->max_cells, (int64_t)d.nx * d.ny * d.nz);
+    (d.fx_pairs ? c->lc.any_fixed : c->lc.any_loops) = true;
     if (d.flags & SPH_SN_LITERAL) c->lc.any_literal = true;
     if (d.flags & SPH_COLLISION) c->lc.any_collision = true;
     if (d.flags & SPH_PFILTER) c->lc.any_filter = true;

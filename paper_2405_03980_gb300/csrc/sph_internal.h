@@ -63,6 +63,8 @@ struct InstDev {
   fx::Unit fx_unit;
   int64_t fx_Hz;
   uint64_t fx_near, fx_width, fx_far;
+  int64_t fx_pairs;               // whether the pair pass is in fixed point (else FP64 loops)
+  double rho_light;               // densities below it are summed in FP64 (0: none)
   float cut2f_margin;             // FP32 prefilter bound (>= every FP64 neighbour)
   float Hzf, half_Hzf;
   int32_t nx, ny, nz;             // cells per axis (ghost ring except periodic z)
@@ -248,7 +250,8 @@ struct NbrWs {
   // each in sorted order.
   uint32_t* parts;
   uint32_t* lead;       // leading zeros of the largest t = 1 - r / 2h of each class, 8 bits
-                        // each, 32 at most, for the pair pass's scales
+                        // each, 32 at most, for the pair pass's scales; the top bit:
+                        // not in fixed point there (InstDev::fx_pairs)
   uint32_t* order;
   uint32_t* part;       // per-tile counts of the partition, then its totals
   float4* posf;         // FP32 copy of sorted positions (FP64-form prefilter)

@@ -155,3 +155,31 @@ def test_lists_of_a_thousand_neighbours():
     print(per_particle_check(sim.state_arrays(), c, 0))
     assert neighbours_equal(sim, c)
     sim.close()
+
+
+@pytest.mark.parametrize("ratio", [1e-7, 1e-3, 0.2, 6.0, 1e4])
+@pytest.mark.parametrize("kind", ["pairs", "one unlike"])
+def test_species_of_different_mass(kind, ratio):
+    """Densities, forces and torques where the species' masses differ: a light
+    particle's density can hang on the W shape of one heavy neighbour, volumes
+    and pressures differ by the ratio and its square.  Where FP64 operations
+    form the shapes, r to 1.5 of 2^-53 gives W 6 / t and two more of the
+    products, the density enters V and P / rho^2 of both partners: 24 / t in
+    all (2^-48 / t allows 32), t the smallest of the group; the coefficients'
+    forty operations beside it."""
+    t = 10.0 ** np.random.default_rng(2).uniform(-3.0, -0.3, 900)
+    pos, sp, m, half = sites(kind, t, 4)
+    x = pos.reshape(-1, m, 3)
+    near = 1 - np.linalg.norm(x[:, :, None] - x[:, None], axis=-1) / 2.6
+    t = np.repeat(np.where(near > 0, near, 1.0).min((1, 2)), m)
+    c = box_of(pos, sp, half, mass_ratio=ratio)
+    sim = sim_of(c)
+    st = sim.state_arrays()
+    acc, sa, dsp, sd = exact_sites(c, m)
+    for f, ref, s in (("acc", acc, sa), ("dspin", dsp, sd)):
+        e = np.linalg.norm((st[f] - ref).astype(float), axis=1)
+        rows = s > 0
+        worst = (e[rows] / s[rows] / (5e-15 + 2.0**-48 / t[rows])).max()
+        print(kind, ratio, f, "largest error over its bound", worst)
+        assert rows.sum() > 200 and worst <= 1.0
+    sim.close()
