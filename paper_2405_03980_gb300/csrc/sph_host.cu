@@ -189,14 +189,16 @@ sph_status derive(const sph_params& p, InstDev& d) {
   // r^2 < (2h)^2 rounds each coordinate difference by up to 2^-53 of the
   // largest coordinate or period and its sums of squares by a few 2^-53; a
   // fixed-point r^2 within fx_band of the cutoff (eight times that, plus its
-  // own few units) is left to the FP64 test, so the sets are the same.  Where
-  // the prefilter lets pairs beyond 1.02 (2h) through (a box of tens of
-  // thousands of supports), every pair is.
+  // own few units) is left to the FP64 test, so the sets are the same.  A pair
+  // vector holds components below 2 (2h): with the prefilter's bound below
+  // 2.8 (2h)^2, the FP32 test passes no pair beyond 1.88 (2h), its coordinates
+  // being off by 0.12 (2h) at most.  Where that does not hold (coordinates of
+  // a million supports), every pair is left to the FP64 test.
   d.fx_unit = fx::make_unit(2.0 * h);
   d.fx_Hz = fx::to_fixed(Hz, d.fx_unit);
   {
     const double rel = ldexp(32.0 + 16.0 * (2.0 * xmax + Hz) / (2.0 * h), -53);
-    const bool ok = (double)d.cut2f_margin < 1.04 * d.cut2 && rel < 1e-3;
+    const bool ok = (double)d.cut2f_margin < 2.8 * d.cut2 && rel < 1e-3;
     const uint64_t band = ok ? 64u + (uint64_t)ldexp(rel, 60) : 0u;
     d.fx_near = fx::kNear2;
     d.fx_width = ok ? fx::kOne2 - band - fx::kNear2 : 0u;

@@ -183,3 +183,17 @@ def test_species_of_different_mass(kind, ratio):
         print(kind, ratio, f, "largest error over its bound", worst)
         assert rows.sum() > 200 and worst <= 1.0
     sim.close()
+
+
+@pytest.mark.parametrize("x0", [2e5, 1e6, 2e6, 5e6])
+def test_boxes_far_from_the_origin(x0):
+    """Where the FP32 prefilter lets pairs through up to 1.1, 1.3, 1.6 and more
+    than 2 supports apart: the fixed-point differences hold them (the last
+    box: every pair by the FP64 test), and the sets are the exact ones."""
+    pos, _, _, sp = synth.periodic_block(8, 8, 8, seed=3, f_v=0.5, jitter=0.3)
+    c = box_of(pos - [4.0, 4.0, 0.0] + [x0, 0.0, 0.0], sp, (8.0, 8.0))
+    c.params = dict(c.params, box_lo=(x0 - 8.0, -8.0, 0.0), box_hi=(x0 + 8.0, 8.0, 8.0))
+    sim = sim_of(c, nbr_cap=128)
+    print(x0, per_particle_check(sim.state_arrays(), c, 0))
+    assert neighbours_equal(sim, c)
+    sim.close()
