@@ -254,10 +254,12 @@ SPH_API sph_status sph_pair_census(sph_ctx* ctx, int32_t inst, int64_t out[5]);
  *    (host or device memory, at least sph_checkpoint_bytes) and leaves the
  *    context unchanged.
  *  - sph_load_checkpoint: restores a checkpoint into ctx, which must have
- *    been created by this library build with the same parameters and counts
- *    (SPH_ERR_ARG otherwise: wrong size, header or instance constants; the
- *    context is then unchanged).  Synchronises.  Stepping on gives, bit for
- *    bit, what the saved context would have given. */
+ *    been created with the same parameters and counts (SPH_ERR_ARG otherwise:
+ *    wrong size, header or instance constants; the context is then
+ *    unchanged).  Synchronises.  Stepping on gives, bit for bit, what the
+ *    saved context would have given.  Files of earlier builds whose particle
+ *    state is laid out the same are taken too; what they step on to differs by
+ *    the rounding of the present passes. */
 SPH_API size_t sph_checkpoint_bytes(const sph_ctx* ctx);
 SPH_API sph_status sph_save_checkpoint(sph_ctx* ctx, void* buf, size_t bytes);
 SPH_API sph_status sph_load_checkpoint(sph_ctx* ctx, const void* buf, size_t bytes);

@@ -1136,6 +1136,32 @@ struct CkptHeader {
 constexpr char kCkptMagic[8] = {'S', 'P', 'H', 'C', 'K', 'P', 'T', '1'};
 constexpr uint32_t kCkptVersion = 2;  // 2: mixed velocity and spin in one record
 
+// Instance records that checkpoints may hold: the present one; its first 688
+// bytes; those without the fixed-point constants and the chunk size.
+constexpr size_t kRecord688 = 688, kRecord624 = 624;
+constexpr size_t kFxBytes = offsetof(InstDev, cut2f_margin) - offsetof(InstDev, fx_unit);
+static_assert(offsetof(InstDev, fx_pairs) == kRecord688 &&
+                  kRecord688 - kFxBytes - sizeof(InstDev::chunk) == kRecord624,
+              "fields are added at the end of InstDev");
+
+// Whether a saved record of rec bytes holds the constants of d.  The reduction
+// chunks are not compared: they follow from the counts, and no state depends
+// on them.
+bool same_constants(const char* saved, size_t rec, InstDev d) {
+  const size_t fx = offsetof(InstDev, fx_unit), fx_end = offsetof(InstDev, cut2f_margin),
+               chunks = offsetof(InstDev, chunk_base), chunk = offsetof(InstDev, chunk),
+               chunks_end = chunk + sizeof d.chunk;
+  const char* now = reinterpret_cast<const char*>(&d);
+  if (rec != kRecord624)
+    return memcmp(saved, now, chunks) == 0 &&
+           memcmp(saved + chunks_end, now + chunks_end, rec - chunks_end) == 0;
+  return memcmp(saved, now, fx) == 0 &&
+         memcmp(saved + fx, now + fx_end, chunks - fx_end) == 0 &&
+         memcmp(saved + chunk - kFxBytes, now + chunks_end, kRecord688 - chunks_end) == 0;
+}
+
+size_t aligned(size_t b) { return (b + kAlign - 1) / kAlign * kAlign; }
+
 }  // namespace
 
 extern "C" {
@@ -1169,22 +1195,30 @@ sph_status sph_save_checkpoint(sph_ctx* c, void* buf, size_t bytes) {
 
 sph_status sph_load_checkpoint(sph_ctx* c, const void* buf, size_t bytes) {
   NvtxRange range("sph_load_checkpoint");
-  if (!c || !buf || bytes < sph_checkpoint_bytes(c)) return SPH_ERR_ARG;
+  if (!c || !buf || bytes < sizeof(CkptHeader)) return SPH_ERR_ARG;
   CK(cudaStreamSynchronize(c->stream));
   const char* in = static_cast<const char*>(buf);
   CkptHeader h;
   CK(cudaMemcpy(&h, in, sizeof h, cudaMemcpyDefault));
   if (memcmp(h.magic, kCkptMagic, sizeof h.magic) != 0 || h.version != kCkptVersion ||
       h.precision != c->precision || h.n_inst != c->n_inst || h.n != c->n ||
-      h.state_bytes != c->state_bytes || (h.cur != 0 && h.cur != 1) ||
-      h.inst_bytes != sizeof(InstDev) * (uint64_t)c->n_inst ||
-      (const char*)c->inst != (const char*)c->state)
+      (h.cur != 0 && h.cur != 1) || (const char*)c->inst != (const char*)c->state)
+    return SPH_ERR_ARG;
+  const size_t n_inst = (size_t)c->n_inst, rec = (size_t)(h.inst_bytes / n_inst);
+  if ((rec != sizeof(InstDev) && rec != kRecord688 && rec != kRecord624) ||
+      h.inst_bytes != rec * n_inst)
+    return SPH_ERR_ARG;
+  // behind the instance records the layouts agree
+  const size_t at_file = aligned(h.inst_bytes), at = aligned(sizeof(InstDev) * n_inst);
+  if (h.state_bytes != c->state_bytes - at + at_file || bytes < sizeof h + h.state_bytes)
     return SPH_ERR_ARG;
   // the instance constants (derived from the parameters and counts) must match
-  std::vector<InstDev> saved((size_t)c->n_inst);
+  std::vector<char> saved(h.inst_bytes);
   CK(cudaMemcpy(saved.data(), in + sizeof h, h.inst_bytes, cudaMemcpyDefault));
-  if (memcmp(saved.data(), c->inst_h.data(), h.inst_bytes) != 0) return SPH_ERR_ARG;
-  CK(cudaMemcpyAsync(c->state, in + sizeof h, c->state_bytes, cudaMemcpyDefault, c->stream));
+  for (size_t k = 0; k < n_inst; ++k)
+    if (!same_constants(saved.data() + k * rec, rec, c->inst_h[k])) return SPH_ERR_ARG;
+  CK(cudaMemcpyAsync((char*)c->state + at, in + sizeof h + at_file, c->state_bytes - at,
+                     cudaMemcpyDefault, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->cur = h.cur;
   c->forces_valid = h.forces_valid != 0;  // the accelerations came with the state

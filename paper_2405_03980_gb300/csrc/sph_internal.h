@@ -63,8 +63,6 @@ struct InstDev {
   fx::Unit fx_unit;
   int64_t fx_Hz;
   uint64_t fx_near, fx_width, fx_far;
-  int64_t fx_pairs;               // whether the pair pass is in fixed point (else FP64 loops)
-  double rho_light;               // densities below it are summed in FP64 (0: none)
   float cut2f_margin;             // FP32 prefilter bound (>= every FP64 neighbour)
   float Hzf, half_Hzf;
   int32_t nx, ny, nz;             // cells per axis (ghost ring except periodic z)
@@ -102,6 +100,11 @@ struct InstDev {
   float skin_cut2_f;              // (2h + skin)^2: the list-build test
   float skin_disp2_f;             // rebuild when |departure|^2 exceeds this (< 0: always)
   float skin_omax_f;              // rebuild when an offset leaves [-omax, L + omax]
+  int64_t fx_pairs;               // FP64 form: whether the pair pass is in fixed point (else
+                                  // FP64 loops)
+  double rho_light;               // densities below it are summed in FP64 (0: none)
+  // (a checkpoint begins with these records: fields are added at the end, and
+  // the records of earlier builds listed beside the loader, sph_host.cu)
 };
 
 // Mutable per-instance scalars that live on the device.
