@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2405_03980_gb300 import _binding as B
 from paper_2405_03980_gb300 import synth
 from test_gpu_fp64 import _cuda, per_particle_check, sim_of  # noqa: F401
 
@@ -197,3 +198,39 @@ def test_boxes_far_from_the_origin(x0):
     print(x0, per_particle_check(sim.state_arrays(), c, 0))
     assert neighbours_equal(sim, c)
     sim.close()
+
+
+def test_partition_tiles_change_no_bit():
+    """The species partition takes larger tiles from 2^20 particles on: a small
+    vessel alone and batched with one that takes the batch past that."""
+    a = synth.cylinder(6.3, 11, Omega=0.13, f_v=0.4, seed=9)
+    b = synth.cylinder(60.0, 100, Omega=0.1, f_v=0.3, seed=10)
+    assert a.n + b.n > 1 << 20
+    solo, both = sim_of(a), sim_of([a, b])
+    solo.step(2)
+    both.step(2)
+    x, y = solo.state_arrays(), both.state_arrays()
+    for k in x:
+        assert np.array_equal(x[k], y[k][:a.n]), k
+    solo.close()
+    both.close()
+
+
+def test_a_batch_keeps_each_instance_on_its_own_pair_pass():
+    """An instance without options equals its solo run bit for bit beside one
+    whose options, and one whose masses, take the FP64 loops."""
+    c = [synth.cylinder(6.3, 11, Omega=0.13, f_v=0.4, seed=9 + k) for k in range(3)]
+    c[1].params = dict(c[1].params, flags=B.SPH_FLAGS_DEFAULT | B.SPH_COLLISION)
+    c[2].params = dict(c[2].params, mass_ratio=20.0)
+    batch = sim_of(c)
+    got, at = batch.state_arrays(), 0
+    for k in c:
+        solo = sim_of(k)
+        for f, x in solo.state_arrays().items():
+            if "flags" in k.params or k.params["mass_ratio"] == 1.0:
+                assert np.array_equal(got[f][at:at + k.n], x), f
+            else:  # (the loops are compiled with the batch's options)
+                assert np.abs(got[f][at:at + k.n] - x).max() <= 1e-13 * np.abs(x).max(), f
+        at += k.n
+        solo.close()
+    batch.close()
