@@ -938,10 +938,10 @@ __global__ void k_pair_records(int64_t n, Fp64Buf b, const InstDev* __restrict__
   }
 }
 
-// One pair in FP64: the force and the spin torque of j on i into out[0..5],
-// and again into out[6..11] if j is a wall.
-__device__ __noinline__ void slow_pair(const Fp64Buf* b, const InstDev* Pp, uint32_t i, uint32_t j,
-                                       int wz, double* out) {
+// One pair in FP64: the force and the spin torque of j on i.  Returns 0 for
+// coincident particles (density only), 2 if j is a wall, else 1.
+__device__ __noinline__ int slow_pair(const Fp64Buf* b, const InstDev* Pp, uint32_t i, uint32_t j,
+                                      int wz, double* f) {
   const InstDev& P = *Pp;
   const dvec4 pi = b->pos[i], vi = b->vel[i], wi = b->spin[i];
   const dvec4 pj = b->pos[j], vj = b->vel[j], wj = b->spin[j];
@@ -950,7 +950,7 @@ __device__ __noinline__ void slow_pair(const Fp64Buf* b, const InstDev* Pp, uint
   if (wz > 0) dz += P.Hz;
   else if (wz < 0) dz -= P.Hz;
   const double r2 = dx * dx + dy * dy + dz * dz;
-  if (!(r2 > 0.0)) return;  // coincident particles: density only
+  if (!(r2 > 0.0)) return 0;
   const double inv_r = rsqrt(r2), r = r2 * inv_r;
   const double t1 = fma(-0.5 * P.inv_h, r, 1.0), t2 = t1 * t1;
   const double F = P.cF * (t2 * t1), W = P.aD * (t2 * t2 * fma(2.0 * P.inv_h, r, 1.0));
@@ -971,7 +971,6 @@ __device__ __noinline__ void slow_pair(const Fp64Buf* b, const InstDev* Pp, uint
   const double sx = 0.5 * (wi.x + wj.x), sy = 0.5 * (wi.y + wj.y), sz = 0.5 * (wi.z + wj.z);
   const double ux = vx + (dy * sz - dz * sy), uy = vy + (dz * sx - dx * sz),
                uz = vz + (dx * sy - dy * sx);
-  double f[6];
   f[0] = (al + aT) * dx;
   f[1] = (al + aT) * dy;
   f[2] = (al + ((fl & SPH_HPROJ) ? 0.0 : aT)) * dz;
@@ -984,11 +983,7 @@ __device__ __noinline__ void slow_pair(const Fp64Buf* b, const InstDev* Pp, uint
     f[4] = -0.5 * bu * (dz * ux - dx * uz);
     f[5] = -0.5 * bu * (dx * uy - dy * ux);
   }
-  const bool wall = is_wall(pj.w);
-  for (int k = 0; k < 6; ++k) {
-    out[k] += f[k];
-    if (wall) out[6 + k] += f[k];
-  }
+  return is_wall(pj.w) ? 2 : 1;
 }
 
 __device__ __forceinline__ int64_t shr(int64_t v, int s) { return v >> (s < 63 ? s : 63); }
@@ -1007,19 +1002,38 @@ struct FxCtx {
 };
 
 // The entries that fixed point does not resolve, in FP64, after the common
-// loops have passed over them, by one lane in the list's order (so that the
-// sums do not depend on the number of lanes): viscous i, the pairs from vv on
-// are of two viscous particles.
+// loops have passed over them: each lane's pair by itself, added up in the
+// list's order (so that the sums do not depend on the number of lanes), every
+// lane left with them: force and torque in out[0..5], the walls' again in
+// out[6..11].  Viscous i: the pairs from vv on are of two viscous particles.
+template <int kL>
 __device__ __noinline__ void slow_walk(int64_t n, int64_t i, uint32_t cnt, uint32_t vv,
                                        const Fp64Buf* b, const InstDev* P, const NbrWs* nw,
                                        const FxCtx* C, double* out) {
-  for (uint32_t t = 0; t < cnt; ++t) {
-    const uint32_t ent = nw->list[nbr_slot(n, i, t)], j = ent & kNbrIndexMask;
-    if ((int64_t)j == i) continue;  // beyond 2h
-    const PairVec v = pair_vec(C->q, nw->posq[j], ent, C->R);
-    const uint64_t r2 = fx::norm2(v.d[0], v.d[1], v.d[2]);
-    if (t >= vv ? r2 - kNearVV < C->width_vv : r2 - C->R.near2 < C->R.width) continue;
-    slow_pair(b, P, (uint32_t)i, j, v.across ? (C->R.bottom ? 1 : -1) : 0, out);
+  const uint32_t lane = threadIdx.x % kL;
+  const uint32_t group = ((1u << kL) - 1u) << (threadIdx.x & 31u & ~(uint32_t)(kL - 1));
+  for (uint32_t t0 = 0; t0 < cnt; t0 += kL) {
+    const uint32_t t = t0 + lane;
+    double f[6];
+    int kind = 0;
+    if (t < cnt) {
+      const uint32_t ent = nw->list[nbr_slot(n, i, t)], j = ent & kNbrIndexMask;
+      const PairVec v = pair_vec(C->q, nw->posq[j], ent, C->R);
+      const uint64_t r2 = fx::norm2(v.d[0], v.d[1], v.d[2]);
+      const bool done = t >= vv ? r2 - kNearVV < C->width_vv : r2 - C->R.near2 < C->R.width;
+      if (!done && (int64_t)j != i)  // (an entry that names i is beyond 2h)
+        kind = slow_pair(b, P, (uint32_t)i, j, v.across ? (C->R.bottom ? 1 : -1) : 0, f);
+    }
+    if (!__any_sync(group, kind)) continue;
+    for (int l = 0; l < kL; ++l) {
+      const int k_l = __shfl_sync(group, kind, l, kL);
+      if (!k_l) continue;
+      for (int k = 0; k < 6; ++k) {
+        const double v = __shfl_sync(group, f[k], l, kL);
+        out[k] += v;
+        if (k_l == 2) out[6 + k] += v;
+      }
+    }
   }
 }
 
@@ -1176,6 +1190,8 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   // first walk: the largest exponents, and the largest |v_ij|
   const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
   uint32_t eP = C.q.exps >> 16, ev = C.q.tag >> 16, eh = C.q.exps & 0xFFFFu;
+  const uint32_t own = max(ev, eh);
+  uint32_t em = 4095u;  // the smallest exponent of a pair (0: at rest, which is exact)
   float dv = 0.f;
   const float4 vi = nw.pvel[i];
   for (uint32_t t0 = lane; t0 < cnt; t0 += 4 * kL) {  // four entries' loads in flight
@@ -1199,6 +1215,8 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
       if (t0 + u * kL >= u0) {
         ev = max(ev, m[u].x >> 16);
         eh = max(eh, m[u].y & 0xFFFFu);
+        const uint32_t e = max(own, max(m[u].x >> 16, m[u].y & 0xFFFFu));
+        em = min(em, j[u] != (uint32_t)i && e != 0u ? e : 4095u);
         const float x = fabsf(vi.x - vj[u].x), y = fabsf(vi.y - vj[u].y),
                     z = fabsf(vi.z - vj[u].z);
         dv = fmaxf(dv, fmaxf(x, fmaxf(y, z)));
@@ -1210,6 +1228,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
     eP = max(eP, __shfl_xor_sync(~0u, eP, o));
     ev = max(ev, __shfl_xor_sync(~0u, ev, o));
     eh = max(eh, __shfl_xor_sync(~0u, eh, o));
+    em = min(em, __shfl_xor_sync(~0u, em, o));
     dv = fmaxf(dv, __shfl_xor_sync(~0u, dv, o));
   }
   // 2^E2 above |v_ij| + |r_ij x s| in every component: |v_ij| from its FP32
@@ -1220,9 +1239,11 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const bool still = (ev | eh) == 0u;
   const int E2 = still ? -1020 : max((int)(__float_as_uint(bound) >> 23) - 126, E_h + 2);
   const int E_v1 = max(E_v, E2);
-  // values the scales do not cover (overflow, NaN, FP32 underflow of v_ij)
-  const bool covered = eP < 2047u && ev < 2047u && eh < 2047u &&
-                       bound < 1e30f && (still || bound > 1e-30f);
+  // values the scales do not cover: overflow, NaN, FP32 underflow of v_ij,
+  // pairs a thousand times slower than the fastest (at that ratio the errors
+  // are those of FP64; at 1e10, 1.5e-7 of a particle's pair terms)
+  const bool covered = eP < 2047u && ev < 2047u && eh < 2047u && bound < 1e30f &&
+                       (still || (bound > 1e-30f && E2 - ((int)em - 1022) <= 10));
   {
     C.R = pair_range(P, z_cell(P, cw.skey[i]));
     if (!covered) C.R.width = 0u;
@@ -1300,11 +1321,12 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   if (__any_sync(~0u, any_slow)) {  // the FP64 route
 #pragma unroll
     for (int o = 1; o < kL; o <<= 1) any_slow |= __shfl_xor_sync(~0u, (int)any_slow, o) != 0;
-    if (lane == 0 && any_slow) {
+    if (any_slow) {  // (the same in all lanes of the row)
       double slow[12];
       for (int k = 0; k < 12; ++k) slow[k] = 0.0;
-      slow_walk(n, i, cnt, inv_i ? cnt : na, &b, &P, &nw, &C, slow);
-      for (int k = 0; k < 12; ++k) sums[row][36 + k] = slow[k];
+      slow_walk<kL>(n, i, cnt, inv_i ? cnt : na, &b, &P, &nw, &C, slow);
+      if (lane == 0)
+        for (int k = 0; k < 12; ++k) sums[row][36 + k] = slow[k];
     }
   }
   __syncthreads();

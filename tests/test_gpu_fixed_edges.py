@@ -234,3 +234,18 @@ def test_a_batch_keeps_each_instance_on_its_own_pair_pass():
         at += k.n
         solo.close()
     batch.close()
+
+
+@pytest.mark.parametrize("factor", [1e3, 1e6, 1e10, 1e-10])
+def test_particles_far_faster_than_their_neighbours(factor):
+    """One particle in fifty faster (or slower) than the rest by the factor:
+    forces and torques of the others hang on differences far below the list's
+    largest where the fast ones stand near the cutoff (the oracle is within
+    1e-13 of extended precision on these states)."""
+    pos, vel, spin, sp = synth.periodic_block(10, 10, 8, seed=8, f_v=0.5, jitter=0.2)
+    c = box_of(pos - [5.0, 5.0, 0.0], sp, (10.0, 10.0))
+    c.vel[::50] *= factor
+    c.spin[::50] *= factor
+    sim = sim_of(c)
+    print(factor, per_particle_check(sim.state_arrays(), c, 0))
+    sim.close()
