@@ -211,8 +211,9 @@ BINDING = {
                       "is evaluated from both sides",
     "k_density_mixed": "latency and line lookups of the offset gathers: L1 throughput 78 %, issue "
                        "65 %, 27 warps per SM (ncu, 2,525,900-particle cylinder)",
-    "k_forces_fx": "issue of the fixed-point pair geometry and sums on the integer pipe (issue "
-                   "52 %, L1 53 %, FP64 pipe 7 %; ncu, 2,525,900-particle cylinder): the FMA-rate "
+    "k_forces_fx": "latency of the fixed-point pair geometry and sums on the integer pipe and of "
+                   "the neighbour gathers at 15 warps per SM, nothing saturated (issue 52 %, ALU "
+                   "48 %, L1 51 %, FP64 pipe 6 %; ncu, 2,525,900-particle cylinder): the FMA-rate "
                    "fraction compares the work done and may pass 1; each pair is evaluated from "
                    "both sides",
     "k_density_fp64": "issue of the fixed-point geometry on the integer pipe (issue 68 %, FP64 "

@@ -1,6 +1,6 @@
 // FP64 form of the two-fluid spin-SPH step: every stored field in double
-// precision; the neighbour passes in 62-bit fixed point where that holds more
-// than a double does (sph_fixed.cuh), everything else in double precision.
+// precision; the neighbour passes in 62-bit fixed point where that is at least
+// as exact (sph_fixed.cuh), everything else in double precision.
 //
 // Model (Sec. 2.1, Eqs. 1, 2, 4; Algorithm 1; Sec. 3 boundary set-up):
 //   density   rho_i = sum_j m_j W_ij (self included), Wendland C2, support 2h,
@@ -390,10 +390,10 @@ __device__ __noinline__ double density_light(int64_t n, int64_t i, uint32_t na, 
 //
 // The pair geometry is in fixed point (sph_fixed.cuh): about 120 integer
 // instructions per entry in place of 20 FP64 ones, each of which holds the
-// FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18 of its value
-// (an FP64 evaluation within a few 1.1e-16), and the sum over a list is
-// exact.  20.1M particles: 64.5 ms with FP64 arithmetic, 19.6 ms in fixed
-// point with a thread per particle, 14.0 ms now (bound by issue, 68 %, and the
+// FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18, in units of the
+// self term's (an FP64 evaluation within a few 1.1e-16 of itself), and the sum
+// over a list is exact.  20.1M particles: 64.5 ms with FP64 arithmetic, 19.6 ms in fixed
+// point with a thread per particle, 14.4 ms now (bound by issue, 68 %, and the
 // ALU).  Lists written by the search instead took 10.5 ms here but 7.2 ms more
 // there.  kFilter: some instance uses the pressure filter; the kernel shape of
 // every list entry is then stored beside the list (nw.wsh_d).
@@ -622,7 +622,7 @@ k_pfilter_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ i
 // term alone; unlike species the pressure, interfacial and local-interaction
 // terms (and the latter's spin torque); two viscous particles the pressure,
 // shear and rotational terms and the rotational torque.  The density pass
-// lists a fluid particle's inviscid neighbours first (count_a of them), and
+// lists a fluid particle's inviscid neighbours first (part_inv of them), and
 // the pair pass runs over the fluid particles in species order (all inviscid
 // ones, then all viscous ones), so that each warp walks the two parts of its
 // lists with one specialised loop each: kPathII, kPathIX, kPathVV.
@@ -783,7 +783,8 @@ __device__ __forceinline__ void pair_loop(const PairCtx& C, const InstDev& P, co
 // v_ij), kOptCollision if some instance uses the collision model; the
 // default form (0) has neither and drops both at compile time.  Thread t
 // takes the fluid particle order[t]: t < n_inv are the inviscid ones, and
-// the threads from the fluid count on (the grid covers all n) return.
+// the threads from the fluid count on (the grid covers all n) return, as do
+// those of the instances that k_forces_fx takes.
 template <int BLOCK, int kOpt>
 __global__ void __launch_bounds__(BLOCK, kOpt ? 512 / BLOCK : 0)
 k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst, CellWs cw,
@@ -863,12 +864,14 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 
 // ----------------------------------------------- pair pass in fixed point
 //
-// The default form's pair pass (neither the literal F_sn nor the collision
-// model).  An FP64 operation holds its pipe for 64 issue slots on this part
-// (two thread operations per SM and clock), so the class loops above, 23 to
-// 79 of them per pair, ran 89 % FP64-pipe busy.  Here a pair's vectors are
-// 64-bit fixed point and the sums 96-bit, on the integer pipe; FP64 is left
-// to the coefficients of the finished sums.
+// The pair pass of the instances with neither the literal F_sn nor the
+// collision model, whose species masses are within a factor of eight
+// (InstDev::fx_pairs; the others take the class loops above).  An FP64
+// operation holds its pipe for 64 issue slots on this part (two thread
+// operations per SM and clock), so the class loops, 23 to 79 of them per pair,
+// run 89 % FP64-pipe busy.  Here a pair's vectors are 64-bit fixed point and
+// the sums 96-bit, on the integer pipe; FP64 is left to the coefficients of
+// the finished sums.
 //
 // Scales.  The geometry is in units of 2h (sph_fixed.cuh).  Velocities,
 // h times the spins and P / rho^2 come as mantissas at each particle's own
@@ -888,24 +891,30 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 //
 // kL lanes take a particle's entries in turn, two to eight of them (warps of 16
 // or 8 particles diverge less than warps of 32, and small vessels spread over
-// more warps; see kPairLanes4); their sums are added by shuffles and the block's first threads finish one
-// particle each, so the FP64 instructions of the end are issued by full
-// warps.  The wall neighbours stand at the end of the list and are summed by
-// themselves: their force and torque give the wall torque.  A pair that fixed
-// point does not resolve (see fx_near; two viscous particles closer than
-// 2h / 8; values outside the range the scales cover, NaN among them) is
-// evaluated in FP64 by slow_walk.
+// more warps; see kPairLanes4); their sums are added by shuffles and the
+// block's first threads finish one particle each, so the FP64 instructions of
+// the end are issued by full warps.  The wall neighbours stand at the end of
+// the list and are summed by themselves: their force and torque give the wall
+// torque.  A pair that fixed point does not resolve (see fx_near; two viscous
+// particles closer than 2h / 8) and every pair of a list that the scales do
+// not cover (velocities more than 2^10 apart, overflow, NaN) is evaluated in
+// FP64 by slow_walk.
 //
-// Measured against a 64-bit-mantissa evaluation (vessels of 9,000 to 23,000
-// particles, 0 to 300 steps): relative L2 error of the acceleration 8e-16 to
-// 6e-15 (FP64 loops 3e-15 to 3e-14), of the spin change 2.0e-16 to 2.4e-16
-// (4.1e-16 to 8.1e-16), of the density 7e-17 (3.6e-16).  20.1M particles:
-// 134.3 ms before, 37.4 ms now.
+// Measured against a 64-bit-mantissa evaluation (vessels of 10,800 to 33,280
+// particles: lattices, up to 300 steps, jitter of 0.3 dx at f_v = 0.01, starts
+// from rest): largest error per particle relative to its pair terms, of the
+// acceleration 1.2e-15 to 7.9e-15 (FP64 loops 5.4e-15 to 5.9e-14), of the spin
+// change 3.5e-16 to 1.5e-14 (1.0e-15 to 2.7e-11), of the density 2.4e-16 to
+// 3.0e-16 (1.4e-15 to 2.4e-15).  20.1M particles: 134.3 ms in FP64, 39.7 ms
+// here (37.6 ms with positions jittered by 0.3 dx).  Nothing is saturated: at
+// 15.3 warps per SM (128 registers) issue is 52 % busy, the ALU 48 %, the FMA
+// pipe's multiplier 45 %, L1 51 %; the warps wait on their chains of integer
+// products (2.0 warps per issue) and on their gathers (1.7).
 
 // Particles below which eight and four lanes take a list, else two: more lanes
 // fill the GPU sooner, fewer spend less on adding up (pair pass with 8 / 4 / 2
-// lanes: 10,800 particles 58 / 73 / 124 us; with 4 / 2 169,000 369 / 376 us, 348,000 735 /
-// 718 us, 2.5M 5.23 / 4.80 ms).
+// lanes: 10,800 particles 59 / 78 / 120 us, 132,000 331 / 303 / 312 us, 169,000
+// 421 / 379 / 385 us, 335,000 838 / 722 / 702 us, 2.6M 6.59 / 5.44 / 4.98 ms).
 constexpr int64_t kPairLanes8 = 1 << 15;
 constexpr int64_t kPairLanes4 = 1 << 18;
 constexpr u64 kNearVV = 1ull << 54;  // (2h / 8)^2, the range of fx::recip

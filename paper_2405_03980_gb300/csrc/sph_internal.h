@@ -215,10 +215,6 @@ struct CellWs {
 // writes one bit per candidate of its cell: word k of particle i, at
 // mask[k * n + i], covers candidates 32k .. 32k + 31, from which the reused
 // lists (mixed form) and the density pass's lists (FP64 form) are built.
-// the fields of NbrWs::parts
-__host__ __device__ __forceinline__ uint32_t part_inv(uint32_t p) { return p & 0x7FFu; }
-__host__ __device__ __forceinline__ uint32_t part_vis(uint32_t p) { return (p >> 11) & 0x7FFu; }
-__host__ __device__ __forceinline__ uint32_t part_dead(uint32_t p) { return p >> 22; }
 constexpr uint32_t kNbrIndexBits = 26;
 constexpr uint32_t kNbrIndexMask = (1u << kNbrIndexBits) - 1u;
 constexpr int64_t kMaxParticles = (int64_t)1 << kNbrIndexBits;  // 67,108,864
@@ -240,6 +236,11 @@ constexpr int kOptCollision = 2;  // collision model (SPH_COLLISION)
 __host__ __device__ __forceinline__ int64_t nbr_slot(int64_t n, int64_t i, uint32_t t) {
   return (((int64_t)(t >> 3) * n + i) << 3) + (int64_t)(t & 7u);
 }
+
+// The fields of NbrWs::parts.
+__host__ __device__ __forceinline__ uint32_t part_inv(uint32_t p) { return p & 0x7FFu; }
+__host__ __device__ __forceinline__ uint32_t part_vis(uint32_t p) { return (p >> 11) & 0x7FFu; }
+__host__ __device__ __forceinline__ uint32_t part_dead(uint32_t p) { return p >> 22; }
 
 struct NbrWs {
   uint32_t* list;       // neighbour entries, layout above

@@ -14,10 +14,11 @@
 // order, which is the neighbour order of the lists it writes for the pair
 // pass.
 //
-// Mixed form: the test is exact, r^2 < (2h)^2 in FP32 on the pair vector
-// (c_i - c_j) L + (o_i - o_j), which every later use of the entry recomputes
-// bit for bit; the test of (j, i) negates that of (i, j), so the neighbour
-// sets are symmetric.  Table entries carry the cell-displacement code.
+// Mixed form: the test is exact, r^2 < (2h + skin)^2 in FP32 on the pair vector
+// (c_i - c_j) L + (o_i - o_j) of the build; the test of (j, i) negates that of
+// (i, j), so the lists are symmetric.  Table entries carry the
+// cell-displacement code.  The density pass tests r < 2h on the current
+// offsets.
 // FP64 form (k_cell_search64): an FP32 prefilter on rounded absolute positions
 // (the periodic image in z taken per candidate) against a widened bound, a
 // superset of the FP64 neighbours, which the density pass tests exactly.  The
