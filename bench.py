@@ -123,20 +123,20 @@ SEARCH_ALGO_BYTES_PER_PARTICLE = {"fp64": 16, "mixed": 16}
 # only while the kernel's sources hash to the values recorded with it; after
 # any change the roofline reports traffic null until it is re-measured.
 DRAM_BYTES_PER_PARTICLE = {
-    "k_cell_search": (222.6, {"sph_search.cu": "764fce7b782403f0",
-                              "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_cell_search64": (194.9, {"sph_search.cu": "764fce7b782403f0",
-                                "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_density_mixed": (774.4, {"sph_mixed.cu": "5582ad1e7bfa79a9",
-                                "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_forces_mixed": (417.4, {"sph_mixed.cu": "5582ad1e7bfa79a9",
-                               "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_density_fp64": (657.8, {"sph_fp64.cu": "a5ab8bffef1ad845",
-                               "sph_fixed.cuh": "da7c2d15ff1f6f0b",
-                               "sph_internal.h": "286e6bd5d58bd3e4"}),
-    "k_forces_fx": (952.7, {"sph_fp64.cu": "a5ab8bffef1ad845",
-                            "sph_fixed.cuh": "da7c2d15ff1f6f0b",
-                            "sph_internal.h": "286e6bd5d58bd3e4"}),
+    "k_cell_search": (222.6, {"sph_search.cu": "d578a7128560e60d",
+                              "sph_internal.h": "8a2e120937f82f0c"}),
+    "k_cell_search64": (194.7, {"sph_search.cu": "d578a7128560e60d",
+                                "sph_internal.h": "8a2e120937f82f0c"}),
+    "k_density_mixed": (774.2, {"sph_mixed.cu": "5582ad1e7bfa79a9",
+                                "sph_internal.h": "8a2e120937f82f0c"}),
+    "k_forces_mixed": (417.5, {"sph_mixed.cu": "5582ad1e7bfa79a9",
+                               "sph_internal.h": "8a2e120937f82f0c"}),
+    "k_density_fp64": (661.6, {"sph_fp64.cu": "0373530b7431d5b2",
+                               "sph_fixed.cuh": "c42db3bbc3948502",
+                               "sph_internal.h": "8a2e120937f82f0c"}),
+    "k_forces_fx": (963.9, {"sph_fp64.cu": "0373530b7431d5b2",
+                            "sph_fixed.cuh": "c42db3bbc3948502",
+                            "sph_internal.h": "8a2e120937f82f0c"}),
     "k_forces_fp64": (None, {}),
 }
 

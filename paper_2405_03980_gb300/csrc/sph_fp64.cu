@@ -393,7 +393,7 @@ __device__ __noinline__ double density_light(int64_t n, int64_t i, uint32_t na, 
 // FP64 pipe for 64 issue slots.  A W shape is within 7.5e-18, in units of the
 // self term's (an FP64 evaluation within a few 1.1e-16 of itself), and the sum
 // over a list is exact.  20.1M particles: 64.5 ms with FP64 arithmetic, 19.6 ms in fixed
-// point with a thread per particle, 14.4 ms now (bound by issue, 68 %, and the
+// point with a thread per particle, 14.3 ms now (bound by issue, 68 %, and the
 // ALU).  Lists written by the search instead took 10.5 ms here but 7.2 ms more
 // there.  kFilter: some instance uses the pressure filter; the kernel shape of
 // every list entry is then stored beside the list (nw.wsh_d).
@@ -905,8 +905,8 @@ k_forces_fp64(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ in
 // from rest): largest error per particle relative to its pair terms, of the
 // acceleration 1.2e-15 to 7.9e-15 (FP64 loops 5.4e-15 to 5.9e-14), of the spin
 // change 3.5e-16 to 1.5e-14 (1.0e-15 to 2.7e-11), of the density 2.4e-16 to
-// 3.0e-16 (1.4e-15 to 2.4e-15).  20.1M particles: 134.3 ms in FP64, 39.7 ms
-// here (37.6 ms with positions jittered by 0.3 dx).  Nothing is saturated: at
+// 3.0e-16 (1.4e-15 to 2.4e-15).  20.1M particles: 134.3 ms in FP64, 39.5 ms
+// here (38.2 ms with positions jittered by 0.3 dx).  Nothing is saturated: at
 // 15.3 warps per SM (128 registers) issue is 52 % busy, the ALU 48 %, the FMA
 // pipe's multiplier 45 %, L1 51 %; the warps wait on their chains of integer
 // products (2.0 warps per issue) and on their gathers (1.7).
