@@ -1200,7 +1200,8 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
   const uint32_t u0 = inv_i ? na : 0u;  // from here on the entries see the velocities
   uint32_t eP = C.q.exps >> 16, ev = C.q.tag >> 16, eh = C.q.exps & 0xFFFFu;
   const uint32_t own = max(ev, eh);
-  uint32_t em = 4095u;  // the smallest exponent of a pair (0: at rest, which is exact)
+  uint32_t em = 4095u;  // the smallest exponent of a pair (at rest too: the products of a zero
+                        // come out as a unit)
   float dv = 0.f;
   const float4 vi = nw.pvel[i];
   for (uint32_t t0 = lane; t0 < cnt; t0 += 4 * kL) {  // four entries' loads in flight
@@ -1225,7 +1226,7 @@ k_forces_fx(int64_t n, Fp64Buf b, Fp64Fields f, const InstDev* __restrict__ inst
         ev = max(ev, m[u].x >> 16);
         eh = max(eh, m[u].y & 0xFFFFu);
         const uint32_t e = max(own, max(m[u].x >> 16, m[u].y & 0xFFFFu));
-        em = min(em, j[u] != (uint32_t)i && e != 0u ? e : 4095u);
+        em = min(em, j[u] != (uint32_t)i ? e : 4095u);
         const float x = fabsf(vi.x - vj[u].x), y = fabsf(vi.y - vj[u].y),
                     z = fabsf(vi.z - vj[u].z);
         dv = fmaxf(dv, fmaxf(x, fmaxf(y, z)));

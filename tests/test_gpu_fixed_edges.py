@@ -249,3 +249,29 @@ def test_particles_far_faster_than_their_neighbours(factor):
     sim = sim_of(c)
     print(factor, per_particle_check(sim.state_arrays(), c, 0))
     sim.close()
+
+
+def test_fluid_at_rest_beside_walls_that_turn():
+    """A start from rest: among the unlike neighbours of a particle near the
+    wall the fluid ones do not move, and the torque hangs on a wall particle
+    that may stand at the cutoff (the oracle's shapes there are good to
+    8 / t of 2^-53, which allows 1e-12 down to t = 0.001)."""
+    c = synth.cylinder(7.0, 11, Omega=0.18, f_v=0.02, seed=3, jitter=0.35, dummy_layers=2)
+    fl = c.species < 2
+    c.vel[fl] = 0.0
+    d = c.pos[fl][:, None] - c.pos[~fl][None]
+    d[..., 2] -= 11.0 * np.round(d[..., 2] / 11.0)
+    t = 1 - np.sqrt((d * d).sum(-1)) / 2.6
+    nearest = t.max(1)
+    assert ((nearest > 1e-3) & (nearest < 0.02)).sum() > 5
+    sim = sim_of(c)
+    st = sim.state_arrays()
+    p = oracle.make_params(c.params)
+    rho, P = oracle.density(p, c.pos, c.species)
+    _, dsp, _, sc = oracle.forces(p, c.pos, c.vel, c.spin, c.species, rho, P, scale=True)
+    e = np.linalg.norm(st["dspin"][fl] - dsp[fl], axis=1)
+    rows = (sc[fl, 1] > 0) & (nearest > 1e-3)
+    print((e[rows] / sc[fl, 1][rows]).max())
+    assert (e[rows] <= 1e-12 * sc[fl, 1][rows]).all()
+    assert (st["dspin"][fl][sc[fl, 1] == 0] == 0).all()
+    sim.close()
