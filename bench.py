@@ -131,10 +131,10 @@ DRAM_BYTES_PER_PARTICLE = {
                                 "sph_internal.h": "8a2e120937f82f0c"}),
     "k_forces_mixed": (417.5, {"sph_mixed.cu": "5582ad1e7bfa79a9",
                                "sph_internal.h": "8a2e120937f82f0c"}),
-    "k_density_fp64": (661.6, {"sph_fp64.cu": "0373530b7431d5b2",
+    "k_density_fp64": (661.6, {"sph_fp64.cu": "7f9cc0c021941ea4",
                                "sph_fixed.cuh": "c42db3bbc3948502",
                                "sph_internal.h": "8a2e120937f82f0c"}),
-    "k_forces_fx": (963.9, {"sph_fp64.cu": "0373530b7431d5b2",
+    "k_forces_fx": (963.9, {"sph_fp64.cu": "7f9cc0c021941ea4",
                             "sph_fixed.cuh": "c42db3bbc3948502",
                             "sph_internal.h": "8a2e120937f82f0c"}),
     "k_forces_fp64": (None, {}),
